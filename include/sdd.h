@@ -231,6 +231,13 @@ int32_t sdd_debug_gemm_bf16(const void* A, int64_t a_rows_capacity, const void* 
                             int32_t use_tensor_cores, int32_t* status_word, void* stream, const void* A_lo,
                             void* out_lo);
 
+/* Diagnostic: the library's fp32 GEMM on its own,  C[M, N] = A[M, K] W[N, K]^T  (the contractions of the fp32
+ * configuration).  A fp32, dense [a_rows_capacity, K] of which the first M rows are used; W fp32 [N, K]; bias fp32 [N] or
+ * null; out fp32, row stride ldc >= N; epilogue as above (all outputs are fp32 here).  K a multiple of 4; A and W 16-byte
+ * aligned; W must be complete in memory when the call is made. */
+int32_t sdd_debug_gemm_f32(const float* A, int64_t a_rows_capacity, const float* W, const float* bias, int32_t M, int32_t N,
+                           int32_t K, int32_t epilogue, float* out, int32_t ldc, int32_t* status_word, void* stream);
+
 /* Diagnostic: the library's bf16 tensor-core attention on its own (d_head = 64), as used inside both
  * networks' blocks: out = softmax(Q K^T / 8 [+ mask]) V per head.
  *   q   device bf16 [q_rows_total, q_ld]; head h occupies columns q_col0 + 64 h .. ; sequence b owns rows

@@ -32,7 +32,7 @@ EXPORTS = [
     "sdd_workspace_bytes", "sdd_create", "sdd_reset", "sdd_draft_begin", "sdd_draft_step", "sdd_draft",
     "sdd_verify_accept", "sdd_step", "sdd_ar_step", "sdd_sps_workspace_bytes", "sdd_sps_attach", "sdd_sps_step",
     "sdd_progress", "sdd_accept_scratch_bytes", "sdd_accept_logits",
-    "sdd_accept_logits_static", "sdd_debug_gemm_bf16", "sdd_debug_attention_bf16", "sdd_debug_wait_timeout",
+    "sdd_accept_logits_static", "sdd_debug_gemm_bf16", "sdd_debug_gemm_f32", "sdd_debug_attention_bf16", "sdd_debug_wait_timeout",
     "sdd_tap", "sdd_counters", "sdd_profile_begin", "sdd_profile_end", "sdd_sync_status", "sdd_destroy", "sdd_strerror", "sdd_last_cuda_error",
 ]
 
@@ -86,6 +86,7 @@ def lib() -> C.CDLL:
         L.sdd_accept_logits.argtypes = [vp, vp, vp, i32, i32, i32, f32, f32, u64, u64, vp, vp, vp, vp, vp]
         L.sdd_accept_logits_static.argtypes = [vp, vp, vp, i32, i32, i32, f32, f32, u64, u64, vp, vp, vp, vp]
         L.sdd_debug_gemm_bf16.argtypes = [vp, C.c_int64, vp, vp, i32, i32, i32, i32, vp, i32, i32, i32, vp, vp, vp, vp]
+        L.sdd_debug_gemm_f32.argtypes = [vp, C.c_int64, vp, vp, i32, i32, i32, i32, vp, i32, vp, vp]
         L.sdd_debug_attention_bf16.argtypes = [vp, C.c_int64, i32, i32, vp, C.c_int64, i32, i32, i32, vp, i32, vp, i32, vp,
                                                i32, i32, i32, i32, i32, vp, vp]
         L.sdd_debug_wait_timeout.argtypes = [C.c_int64, vp, vp]
@@ -217,6 +218,15 @@ def sdd_debug_gemm_bf16(A, W, bias, M: int, epilogue: int, out, n_tile: int = 0,
                                      A_lo.data_ptr() if A_lo is not None else None,
                                      out_lo.data_ptr() if out_lo is not None else None),
            "sdd_debug_gemm_bf16")
+
+
+def sdd_debug_gemm_f32(A, W, bias, M: int, epilogue: int, out, status=None, stream=None):
+    """out = epilogue(A[:M] @ W.T + bias) with the library's fp32 GEMM; A [cap, K], W [N, K], out fp32 CUDA tensors."""
+    torch = _torch()
+    st = stream if stream is not None else torch.cuda.current_stream(A.device)
+    _check(lib().sdd_debug_gemm_f32(A.data_ptr(), A.shape[0], W.data_ptr(), bias.data_ptr() if bias is not None else None, M,
+                                    W.shape[0], A.shape[1], epilogue, out.data_ptr(), out.stride(0),
+                                    status.data_ptr() if status is not None else None, st.cuda_stream), "sdd_debug_gemm_f32")
 
 
 def sdd_debug_attention_bf16(q, q_col0, k, k_col0, k_rows_per_seq, vt, out, ctx_len, batch, n_head, gamma, mode,

@@ -269,12 +269,15 @@ static int gemm(sdd_ctx* c, int cat, const void* A, size_t a_elems, const void* 
   if (M <= 0) return SDD_OK;
   ProfScope prof(c, cat);
   c->launches++;
-  if (std::is_same<T, __nv_bfloat16>::value && !c->force_simt) {
+  if constexpr (std::is_same<T, float>::value) {
+    SDD_CUDA(launch_gemm_f32((const float*)A, (long long)(a_elems / (size_t)K), (const float*)W, bias, (int)M, N, K, epi,
+                             (float*)out, ldc, &c->B.rs->status, c->st, skip));
+  } else if (!c->force_simt) {
     SDD_CUDA(launch_gemm_tc((const __nv_bfloat16*)A, (long long)(a_elems / (size_t)K), (const __nv_bfloat16*)W, bias, (int)M,
                             N, K, epi, out, ldc, c->bn_hint, &c->B.rs->status, c->st, qd, (const __nv_bfloat16*)A_lo, out_lo, skip,
                             c->head_stats ? stats : nullptr, stats_chunks));
   } else {
-    SDD_CUDA(launch_gemm_simt<T>((const T*)A, K, (const T*)W, bias, (int)M, N, K, epi, out, ldc, c->st, skip));
+    SDD_CUDA(launch_gemm_simt((const T*)A, K, (const T*)W, bias, (int)M, N, K, epi, out, ldc, c->st, skip));
   }
   return SDD_OK;
 }
@@ -635,6 +638,8 @@ int32_t sdd_create(const sdd_model* target, const sdd_model* drafter, const sdd_
   if (c->P.dtype == SDD_BF16) {   // before anything can be captured into a graph
     SDD_CUDA(tc_prepare_gemm());
     SDD_CUDA(tc_prepare_attn());
+  } else {
+    SDD_CUDA(tc_prepare_gemm_f32());
   }
   // the tensor-core attention multiplies masked probabilities (exact zeros) with whatever the V^T cache holds
   // past the valid positions, so that memory must be finite
@@ -988,8 +993,16 @@ int32_t sdd_debug_gemm_bf16(const void* A, int64_t a_rows_capacity, const void* 
     SDD_CUDA(launch_gemm_tc((const __nv_bfloat16*)A, a_rows_capacity, (const __nv_bfloat16*)W, bias, M, N, K, epilogue, out,
                             ldc, n_tile, status_word, st, nullptr, (const __nv_bfloat16*)A_lo, out_lo));
   else
-    SDD_CUDA(launch_gemm_simt<__nv_bfloat16>((const __nv_bfloat16*)A, K, (const __nv_bfloat16*)W, bias, M, N, K, epilogue,
+    SDD_CUDA(launch_gemm_simt((const __nv_bfloat16*)A, K, (const __nv_bfloat16*)W, bias, M, N, K, epilogue,
                                              out, ldc, st));
+  return SDD_OK;
+}
+
+int32_t sdd_debug_gemm_f32(const float* A, int64_t a_rows_capacity, const float* W, const float* bias, int32_t M, int32_t N,
+                           int32_t K, int32_t epilogue, float* out, int32_t ldc, int32_t* status_word, void* stream) {
+  if (!A || !W || !out || M < 1 || N < 1 || K < 4 || (K % 4) != 0 || epilogue < 0 || epilogue > 3) return SDD_E_ARG;
+  if (a_rows_capacity < M || ldc < N) return SDD_E_ARG;
+  SDD_CUDA(launch_gemm_f32(A, a_rows_capacity, W, bias, M, N, K, epilogue, out, ldc, status_word, (cudaStream_t)stream));
   return SDD_OK;
 }
 

@@ -1,13 +1,13 @@
 // CUDA-core GEMM  C[M, N] = A[M, K] * W[N, K]^T  with fused epilogues.
-// This is the contraction of the fp32 configuration (fp32 storage and accumulation, where tensor
-// cores have no fp32 operand type) and a slow cross-check of the bf16 tensor-core GEMM.
+// A slow cross-check of the bf16 tensor-core GEMM.
 #include "sdd_kernels.h"
 
 namespace sdd {
 
 constexpr int SG_BM = 64, SG_BN = 64, SG_BK = 16, SG_THREADS = 256;
 
-template <typename T>
+using T = __nv_bfloat16;
+
 __global__ void __launch_bounds__(SG_THREADS)
 gemm_simt_kernel(const T* __restrict__ A, int lda, const T* __restrict__ W, const float* __restrict__ bias, int M, int N,
                  int K, int epi, void* __restrict__ out, int ldc, const int* __restrict__ skip) {
@@ -59,18 +59,12 @@ gemm_simt_kernel(const T* __restrict__ A, int lda, const T* __restrict__ W, cons
   }
 }
 
-template <typename T>
 cudaError_t launch_gemm_simt(const T* A, int lda, const T* W, const float* bias, int M, int N, int K, int epi, void* out,
                              int ldc, cudaStream_t st, const int* skip) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   dim3 grid((N + SG_BN - 1) / SG_BN, (M + SG_BM - 1) / SG_BM);
-  launch_k(gemm_simt_kernel<T>, dim3(grid), dim3(SG_THREADS), 0, st, A, lda, W, bias, M, N, K, epi, out, ldc, skip);
+  launch_k(gemm_simt_kernel, dim3(grid), dim3(SG_THREADS), 0, st, A, lda, W, bias, M, N, K, epi, out, ldc, skip);
   return cudaGetLastError();
 }
-
-template cudaError_t launch_gemm_simt<float>(const float*, int, const float*, const float*, int, int, int, int, void*, int,
-                                             cudaStream_t, const int*);
-template cudaError_t launch_gemm_simt<__nv_bfloat16>(const __nv_bfloat16*, int, const __nv_bfloat16*, const float*, int,
-                                                     int, int, int, void*, int, cudaStream_t, const int*);
 
 }  // namespace sdd

@@ -116,11 +116,16 @@ template <typename T>
 cudaError_t launch_kv_append(const T* qkv, T* cache, const int* ctx_len, int batch, int rows_per_seq, int mode, int n_ctx,
                              int d, cudaStream_t st);
 
-// ---- GEMM (sdd_gemm_simt.cu, sdd_gemm_tc.cu) ------------------------------------------------
+// ---- GEMM (sdd_gemm_simt.cu, sdd_gemm_f32.cu, sdd_gemm_tc.cu) -------------------------------
 // C[M, N] = A[M, K] * W[N, K]^T; A row stride lda, W row stride K, out row stride ldc.
-template <typename T>
-cudaError_t launch_gemm_simt(const T* A, int lda, const T* W, const float* bias, int M, int N, int K, int epi, void* out,
-                             int ldc, cudaStream_t st, const int* skip = nullptr);
+// bf16 on the CUDA cores: the cross-check of the tensor-core kernels
+cudaError_t launch_gemm_simt(const __nv_bfloat16* A, int lda, const __nv_bfloat16* W, const float* bias, int M, int N, int K,
+                             int epi, void* out, int ldc, cudaStream_t st, const int* skip = nullptr);
+
+// fp32 operands, products and sums (tensor cores on exact bf16 triples, see sdd_gemm_f32.cu); A is a dense [a_cap, K]
+// buffer of which M rows are used; K a multiple of 4, A and W 16-byte aligned
+cudaError_t launch_gemm_f32(const float* A, long long a_cap, const float* W, const float* bias, int M, int N, int K, int epi,
+                            float* out, int ldc, int* status, cudaStream_t st, const int* skip = nullptr);
 
 // bf16 tensor-core GEMM (tcgen05 / TMEM / TMA).  A is a dense [a_cap, K] buffer of which M rows are used;
 // bn_hint selects the N tile (0 = choose); a bounded wait that expires sets *status = DEV_TIMEOUT.
@@ -138,6 +143,7 @@ cudaError_t launch_wait_timeout_probe(long long limit_cycles, int* status, cudaS
 
 // one-time set-up of the tensor-core kernels (dynamic shared-memory limits); also done lazily on first launch
 cudaError_t tc_prepare_gemm();
+cudaError_t tc_prepare_gemm_f32();
 cudaError_t tc_prepare_attn();
 
 // bf16 tensor-core attention, d_head = 64 (sdd_attn_tc.cu).  q / k are row-major tensors with the heads side by

@@ -14,6 +14,19 @@ constexpr long long WAIT_LIMIT_CYCLES = 2000000000ll;   // about one second
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// One lane of a converged warp.  Instructions that take their operands from uniform registers (tcgen05.mma / commit, TMA)
+// have to sit behind this rather than behind "lane == 0": the compiler then knows that one thread issues them, and emits
+// them straight; otherwise it wraps each in a loop over the lanes that might be active.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\t"
+      "elect.sync _|P, 0xffffffff;\n\t"
+      "selp.b32 %0, 1, 0, P;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
