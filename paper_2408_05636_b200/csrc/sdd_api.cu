@@ -641,6 +641,7 @@ int32_t sdd_create(const sdd_model* target, const sdd_model* drafter, const sdd_
   } else {
     SDD_CUDA(tc_prepare_gemm_f32());
   }
+  SDD_CUDA(prepare_attn());
   // the tensor-core attention multiplies masked probabilities (exact zeros) with whatever the V^T cache holds
   // past the valid positions, so that memory must be finite
   SDD_CUDA(cudaMemsetAsync(c->B.kv, 0, (size_t)c->P.n_layer * params->batch * c->P.n_ctx * 2 * c->P.d * c->D.esize, c->st));

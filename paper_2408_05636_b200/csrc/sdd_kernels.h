@@ -156,6 +156,7 @@ cudaError_t launch_attn_tc(const __nv_bfloat16* q, long long q_rows_total, int q
                            const int* skip = nullptr);
 
 // ---- attention (sdd_attn.cu) ----------------------------------------------------------------
+cudaError_t prepare_attn();   // one-time set-up, as above
 // drafter: every row of a sequence attends to rows 0 .. ctx_len[b] + gamma - 1 of the same sequence
 template <typename T>
 cudaError_t launch_attn_bidir(const T* qkv, T* out, const int* ctx_len, int batch, int gamma, int L_cap, int n_head,
