@@ -633,8 +633,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   // skip flag only decides whether to fetch ahead; a stale value costs time, not correctness.
   constexpr uint32_t W_BYTES = (SWAP ? BM : BN) * BK * 2;
   int n_pre = 0;
-  if (threadIdx.x == 0 && (skip == nullptr || *reinterpret_cast<const volatile int*>(skip) == 0)) {
-    n_pre = min(num_kb, STAGES);
+  if (warp == 0 && (skip == nullptr || *reinterpret_cast<const volatile int*>(skip) == 0)) n_pre = min(num_kb, STAGES);
+  n_pre = __shfl_sync(0xffffffffu, n_pre, 0);
+  if (warp == 0 && elect_one()) {
     for (int kb = 0; kb < n_pre; ++kb) {
       mbar_expect_tx_only(full_bar(kb), W_BYTES);
       const uint32_t sa = base + kb * STAGE_BYTES;
@@ -642,12 +643,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       else tma_load_2d(sa + BM * BK * 2, &map_b, full_bar(kb), (kb0 + kb) * BK, n0);
     }
   }
+  __syncwarp();
   pdl_launch_dependents();
   pdl_wait();
   // The activation tiles of the stages whose weight tiles are already on their way go out at once, before the skip
   // flag has even been read (one L2 round trip that would otherwise sit in front of the first operand tile of every
   // launch of a drafter evaluation); if the evaluation turns out to be skipped the tiles are waited for and dropped.
-  if (threadIdx.x == 0) {
+  if (warp == 0 && elect_one()) {
     for (int kb = 0; kb < n_pre; ++kb) {
       const uint32_t sa = base + kb * STAGE_BYTES;
       mbar_expect_tx(full_bar(kb), (uint32_t)STAGE_BYTES - W_BYTES);
@@ -656,48 +658,50 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       if (HILO) tma_load_2d(sa + LO_OFF, &map_lo, full_bar(kb), (kb0 + kb) * BK, SWAP ? n0 : m0);
     }
   }
+  __syncwarp();
   // launches of a drafter evaluation do nothing when the evaluation is skipped (they still free their TMEM below)
   const bool active = skip == nullptr || *skip == 0;
 
   if (!active) {
     // tiles fetched ahead must have landed before the CTA gives its shared memory back
-    for (int kb = 0; kb < n_pre; ++kb) {
+    for (int kb = 0; threadIdx.x == 0 && kb < n_pre; ++kb) {
       const long long t0 = clock64();
       while (!mbar_try(full_bar(kb), 0u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
     }
   } else if (warp == 0) {
-    if (lane == 0) {
-      int issued = n_pre;
-      for (int kb = n_pre; kb < num_kb; ++kb) {
-        const int s = kb % STAGES;
-        const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
-        const uint32_t sa = base + s * STAGE_BYTES;
-        if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, status)) break;
+    int issued = n_pre;
+    for (int kb = n_pre; kb < num_kb; ++kb) {
+      const int s = kb % STAGES;
+      const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
+      const uint32_t sa = base + s * STAGE_BYTES;
+      if (!mbar_wait_warp(empty_bar(s), ph ^ 1u, abort_flag, status)) break;
+      if (elect_one()) {
         mbar_expect_tx(full_bar(s), (uint32_t)STAGE_BYTES);
         tma_load_2d(sa, &map_a, full_bar(s), (kb0 + kb) * BK, m0);
         tma_load_2d(sa + BM * BK * 2, &map_b, full_bar(s), (kb0 + kb) * BK, n0);
         if (HILO) tma_load_2d(sa + LO_OFF, &map_lo, full_bar(s), (kb0 + kb) * BK, SWAP ? n0 : m0);
-        issued = kb + 1;
       }
-      if (*abort_flag) {
-        // do not leave while copies into this CTA's shared memory may still be in flight
-        const int first = issued > STAGES ? issued - STAGES : 0;
-        for (int kb = first; kb < issued; ++kb) {
-          const long long t0 = clock64();
-          while (!mbar_try(full_bar(kb % STAGES), (uint32_t)(kb / STAGES) & 1u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
-        }
+      __syncwarp();
+      issued = kb + 1;
+    }
+    if (lane == 0 && *abort_flag) {
+      // do not leave while copies into this CTA's shared memory may still be in flight
+      const int first = issued > STAGES ? issued - STAGES : 0;
+      for (int kb = first; kb < issued; ++kb) {
+        const long long t0 = clock64();
+        while (!mbar_try(full_bar(kb % STAGES), (uint32_t)(kb / STAGES) & 1u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = make_idesc<BN>();
-      bool ok = true;
-      for (int kb = 0; kb < num_kb && ok; ++kb) {
-        const int s = kb % STAGES;
-        const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
-        ok = mbar_wait(full_bar(s), ph, abort_flag, status);
-        if (!ok) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    constexpr uint32_t idesc = make_idesc<BN>();
+    bool ok = true;
+    for (int kb = 0; kb < num_kb; ++kb) {
+      const int s = kb % STAGES;
+      const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
+      ok = mbar_wait_warp(full_bar(s), ph, abort_flag, status);
+      if (!ok) break;
+      fence_after_sync();
+      if (elect_one()) {
         const uint32_t sa = base + s * STAGE_BYTES;
         const uint64_t da = make_smem_desc(sa), db = make_smem_desc(sa + BM * BK * 2);
 #pragma unroll
@@ -714,8 +718,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           }
         }
         umma_commit(empty_bar(s));     // frees the stage once these MMAs have read it
+        if (kb == num_kb - 1) umma_commit(tmem_full_bar);
       }
-      if (ok) umma_commit(tmem_full_bar);
+      __syncwarp();
     }
   } else {
     // epilogue warps own TMEM lane quarters (warp id % 4); with two groups, group g = (warp - 2) / 4 takes the chunks
@@ -827,9 +832,12 @@ gemm_tc_persist_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
   // the first ring fill of weight tiles starts before the wait for the kernel ahead (see gemm_tc_kernel)
   constexpr uint32_t W_BYTES = (SWAP ? BM : BN) * BK * 2;
   int n_pre = 0;
-  if (threadIdx.x == 0 && (int)blockIdx.x < n_tiles && (skip == nullptr || *reinterpret_cast<const volatile int*>(skip) == 0)) {
+  if (warp == 0 && (int)blockIdx.x < n_tiles && (skip == nullptr || *reinterpret_cast<const volatile int*>(skip) == 0)) {
     const long long mine = (long long)((n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x) * num_kb;
     n_pre = (int)(mine < STAGES ? mine : STAGES);
+  }
+  n_pre = __shfl_sync(0xffffffffu, n_pre, 0);
+  if (warp == 0 && elect_one()) {
     for (int j = 0; j < n_pre; ++j) {
       const int tile = (int)blockIdx.x + (j / num_kb) * (int)gridDim.x, kb = j % num_kb;
       const int m0 = (n_fastest ? tile / tiles_n : tile % tiles_m) * BM;
@@ -840,66 +848,63 @@ gemm_tc_persist_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
       else tma_load_2d(sa + BM * BK * 2, &map_b, full_bar(j), kb * BK, n0);
     }
   }
+  __syncwarp();
   pdl_launch_dependents();
   pdl_wait();
   const bool active = skip == nullptr || *skip == 0;
 
   if (!active) {
     // weight tiles fetched ahead must have landed before the CTA gives its shared memory back
-    for (int j = 0; j < n_pre; ++j) {
+    for (int j = 0; threadIdx.x == 0 && j < n_pre; ++j) {
       mbar_arrive(full_bar(j));
       const long long t0 = clock64();
       while (!mbar_try(full_bar(j), 0u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
     }
   } else if (warp == 0) {
-    if (lane == 0) {
-      long long it = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-        const int m0 = (n_fastest ? tile / tiles_n : tile % tiles_m) * BM;
-        const int n0 = (n_fastest ? tile % tiles_n : tile / tiles_m) * BN;
-        for (int kb = 0; kb < num_kb; ++kb, ++it) {
-          const int s = (int)(it % STAGES);
-          const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
-          const uint32_t sa = base + s * STAGE_BYTES;
-          if (it < n_pre) {
-            mbar_expect_tx(full_bar(s), (uint32_t)STAGE_BYTES - W_BYTES);    // the weight tile is already on its way
-            if (SWAP) tma_load_2d(sa + BM * BK * 2, &map_b, full_bar(s), kb * BK, n0);
-            else tma_load_2d(sa, &map_a, full_bar(s), kb * BK, m0);
-          } else {
-            if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, status)) { ok = false; break; }
-            mbar_expect_tx(full_bar(s), (uint32_t)STAGE_BYTES);
-            tma_load_2d(sa, &map_a, full_bar(s), kb * BK, m0);
-            tma_load_2d(sa + BM * BK * 2, &map_b, full_bar(s), kb * BK, n0);
-          }
+    long long it = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+      const int m0 = (n_fastest ? tile / tiles_n : tile % tiles_m) * BM;
+      const int n0 = (n_fastest ? tile % tiles_n : tile / tiles_m) * BN;
+      for (int kb = 0; kb < num_kb; ++kb, ++it) {
+        const int s = (int)(it % STAGES);
+        const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
+        const uint32_t sa = base + s * STAGE_BYTES;
+        const bool pre = it < n_pre;           // the weight tile is already on its way
+        if (!pre && !mbar_wait_warp(empty_bar(s), ph ^ 1u, abort_flag, status)) { ok = false; break; }
+        if (elect_one()) {
+          mbar_expect_tx(full_bar(s), (uint32_t)STAGE_BYTES - (pre ? W_BYTES : 0u));
+          if (!pre || !SWAP) tma_load_2d(sa, &map_a, full_bar(s), kb * BK, m0);
+          if (!pre || SWAP) tma_load_2d(sa + BM * BK * 2, &map_b, full_bar(s), kb * BK, n0);
           if (HILO) tma_load_2d(sa + LO_OFF, &map_lo, full_bar(s), kb * BK, SWAP ? n0 : m0);   // the activation side
         }
+        __syncwarp();
       }
-      if (*abort_flag) {
-        // do not leave while copies into this CTA's shared memory may still be in flight
-        for (long long j = it > STAGES ? it - STAGES : 0; j < it; ++j) {
-          const long long t0 = clock64();
-          while (!mbar_try(full_bar((int)(j % STAGES)), (uint32_t)(j / STAGES) & 1u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
-        }
+    }
+    if (lane == 0 && *abort_flag) {
+      // do not leave while copies into this CTA's shared memory may still be in flight
+      for (long long j = it > STAGES ? it - STAGES : 0; j < it; ++j) {
+        const long long t0 = clock64();
+        while (!mbar_try(full_bar((int)(j % STAGES)), (uint32_t)(j / STAGES) & 1u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = make_idesc<BN>();
-      long long it = 0;
-      int i = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++i) {
-        const int buf = i & 1;
-        ok = mbar_wait(tempty_bar(buf), ((uint32_t)(i >> 1) & 1u) ^ 1u, abort_flag, status);   // accumulator drained
+    constexpr uint32_t idesc = make_idesc<BN>();
+    long long it = 0;
+    int i = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++i) {
+      const int buf = i & 1;
+      ok = mbar_wait_warp(tempty_bar(buf), ((uint32_t)(i >> 1) & 1u) ^ 1u, abort_flag, status);   // accumulator drained
+      if (!ok) break;
+      fence_after_sync();
+      const uint32_t acc = tmem_base + (uint32_t)(buf * BN);
+      for (int kb = 0; kb < num_kb; ++kb, ++it) {
+        const int s = (int)(it % STAGES);
+        ok = mbar_wait_warp(full_bar(s), (uint32_t)(it / STAGES) & 1u, abort_flag, status);
         if (!ok) break;
         fence_after_sync();
-        const uint32_t acc = tmem_base + (uint32_t)(buf * BN);
-        for (int kb = 0; kb < num_kb; ++kb, ++it) {
-          const int s = (int)(it % STAGES);
-          ok = mbar_wait(full_bar(s), (uint32_t)(it / STAGES) & 1u, abort_flag, status);
-          if (!ok) break;
-          fence_after_sync();
+        if (elect_one()) {
           const uint32_t sa = base + s * STAGE_BYTES;
           const uint64_t da = make_smem_desc(sa), db = make_smem_desc(sa + BM * BK * 2);
 #pragma unroll
@@ -915,8 +920,9 @@ gemm_tc_persist_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             }
           }
           umma_commit(empty_bar(s));
+          if (kb == num_kb - 1) umma_commit(tfull_bar(buf));
         }
-        if (ok) umma_commit(tfull_bar(buf));
+        __syncwarp();
       }
     }
   } else {
@@ -1035,58 +1041,62 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 
   if (!active) {
   } else if (warp == 0) {
-    if (lane == 0) {
-      long long it = 0;
-      bool ok = true;
-      for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
-        const int m0 = (n_fastest ? tile / tiles_n : tile % tiles_m2) * (2 * BM) + (int)rank * BM;
-        const int n0 = (n_fastest ? tile % tiles_n : tile / tiles_m2) * BN + (int)rank * 128;
-        for (int kb = 0; kb < num_kb; ++kb, ++it) {
-          const int s = (int)(it % STAGES);
-          const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
-          if (!mbar_wait_cluster(empty_bar(s), ph ^ 1u, abort_flag, status)) { ok = false; break; }
+    long long it = 0;
+    bool ok = true;
+    for (int tile = pair; tile < n_tiles && ok; tile += n_pairs) {
+      const int m0 = (n_fastest ? tile / tiles_n : tile % tiles_m2) * (2 * BM) + (int)rank * BM;
+      const int n0 = (n_fastest ? tile % tiles_n : tile / tiles_m2) * BN + (int)rank * 128;
+      for (int kb = 0; kb < num_kb; ++kb, ++it) {
+        const int s = (int)(it % STAGES);
+        const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
+        if (!__all_sync(0xffffffffu, mbar_wait_cluster(empty_bar(s), ph ^ 1u, abort_flag, status))) { ok = false; break; }
+        if (elect_one()) {
           if (leader) mbar_expect_tx(full_bar(s), 2u * (uint32_t)PAIR_STAGE_BYTES);   // both CTAs' bytes
           const uint32_t lf = map_to_cta(full_bar(s), 0u);
           const uint32_t sa = base + s * PAIR_STAGE_BYTES;
           tma_load_2d_pair(sa, &map_a, lf, kb * BK, m0);
           tma_load_2d_pair(sa + BM * BK * 2, &map_b, lf, kb * BK, n0);
         }
+        __syncwarp();
       }
-      if (leader && *abort_flag) {
-        // do not leave while copies into the pair's shared memory may still be in flight (the peer stays until the
-        // cluster barrier at the end, which the leader reaches after this)
-        for (long long j = it > STAGES ? it - STAGES : 0; j < it; ++j) {
-          const long long t0 = clock64();
-          while (!mbar_try_cluster(full_bar((int)(j % STAGES)), (uint32_t)(j / STAGES) & 1u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
-        }
+    }
+    if (lane == 0 && leader && *abort_flag) {
+      // do not leave while copies into the pair's shared memory may still be in flight (the peer stays until the
+      // cluster barrier at the end, which the leader reaches after this)
+      for (long long j = it > STAGES ? it - STAGES : 0; j < it; ++j) {
+        const long long t0 = clock64();
+        while (!mbar_try_cluster(full_bar((int)(j % STAGES)), (uint32_t)(j / STAGES) & 1u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && leader) {
+    if (leader) {
       constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
       long long it = 0;
       int i = 0;
       bool ok = true;
       for (int tile = pair; tile < n_tiles && ok; tile += n_pairs, ++i) {
         const int buf = i & 1;
-        ok = mbar_wait_cluster(tempty_bar(buf), ((uint32_t)(i >> 1) & 1u) ^ 1u, abort_flag, status);   // drained in both CTAs
+        ok = __all_sync(0xffffffffu, mbar_wait_cluster(tempty_bar(buf), ((uint32_t)(i >> 1) & 1u) ^ 1u, abort_flag, status));   // drained in both CTAs
         if (!ok) break;
         fence_after_sync();
         const uint32_t acc = tmem_base + (uint32_t)(buf * BN);
         for (int kb = 0; kb < num_kb; ++kb, ++it) {
           const int s = (int)(it % STAGES);
-          ok = mbar_wait_cluster(full_bar(s), (uint32_t)(it / STAGES) & 1u, abort_flag, status);
+          ok = __all_sync(0xffffffffu, mbar_wait_cluster(full_bar(s), (uint32_t)(it / STAGES) & 1u, abort_flag, status));
           if (!ok) break;
           fence_after_sync();
-          const uint32_t sa = base + s * PAIR_STAGE_BYTES;
-          const uint64_t da = make_smem_desc(sa), db = make_smem_desc(sa + BM * BK * 2);
+          if (elect_one()) {
+            const uint32_t sa = base + s * PAIR_STAGE_BYTES;
+            const uint64_t da = make_smem_desc(sa), db = make_smem_desc(sa + BM * BK * 2);
 #pragma unroll
-          for (int k = 0; k < BK / UMMA_K; ++k)
-            umma_pair(acc, da + (uint64_t)(k * UMMA_K * 2 / 16), db + (uint64_t)(k * UMMA_K * 2 / 16), idesc, (kb > 0 || k > 0) ? 1u : 0u);
-          umma_commit_pair(empty_bar(s));                       // frees the stage in this CTA ...
-          umma_commit_pair(map_to_cta(empty_bar(s), peer));     // ... and in the peer
+            for (int k = 0; k < BK / UMMA_K; ++k)
+              umma_pair(acc, da + (uint64_t)(k * UMMA_K * 2 / 16), db + (uint64_t)(k * UMMA_K * 2 / 16), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+            umma_commit_pair(empty_bar(s));                       // frees the stage in this CTA ...
+            umma_commit_pair(map_to_cta(empty_bar(s), peer));     // ... and in the peer
+            if (kb == num_kb - 1) umma_commit_pair(tfull_bar(buf));
+          }
+          __syncwarp();
         }
-        if (ok) umma_commit_pair(tfull_bar(buf));
       }
     }
   } else {
