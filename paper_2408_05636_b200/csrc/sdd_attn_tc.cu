@@ -137,7 +137,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   // skip flag, whose loads would otherwise sit in front of them (with a key split the first tile of a CTA may not exist,
   // so only unsplit launches do this).  A CTA that turns out to have nothing to do waits for the copies and drops them.
   const bool spec = kv_split == 1;
-  if (spec && threadIdx.x == 0) {
+  if (spec && warp == 0 && elect_one()) {
     mbar_expect_tx(q_full, AT_Q_BYTES);
     tma_load_2d(sQ, &map_q, q_full, prm.q_col0 + h * AT_DH, b * prm.q_rows_per_seq + qt * 128);
     mbar_expect_tx(kv_full(0), AT_STAGE_BYTES);
@@ -145,6 +145,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     tma_load_2d(sVT(0), &map_vt, kv_full(0), 0, b * prm.d + h * AT_DH);
     tma_load_2d(sVT(0) + 64 * 64 * 2, &map_vt, kv_full(0), 64, b * prm.d + h * AT_DH);
   }
+  __syncwarp();
   // a skipped drafter evaluation, or a tile of padding rows only: nothing to do (uniform over the CTA and its cluster)
   bool active = !(prm.skip != nullptr && *prm.skip);
   const int c = active ? prm.ctx_len[b] : 1;
@@ -177,23 +178,27 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
       while (!mbar_try(kv_full(0), 0u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
     }
   } else if (warp == 0) {
-    if (lane == 0 && my_kt > 0) {   // (an unsplit launch that is active has at least one key tile)
-      if (!spec) {
+    if (my_kt > 0) {   // (an unsplit launch that is active has at least one key tile)
+      if (!spec && elect_one()) {
         mbar_expect_tx(q_full, AT_Q_BYTES);
         tma_load_2d(sQ, &map_q, q_full, prm.q_col0 + h * AT_DH, b * prm.q_rows_per_seq + q0);
       }
+      __syncwarp();
       int issued = spec ? 1 : 0;
       for (int it = issued; it < my_kt; ++it) {
         const int t = kv_rank + it * kv_split;      // key tile; `it` counts this CTA's iterations (stages, phases)
         const int s = it % AT_KV_STAGES;
-        if (!mbar_wait(kv_empty(s), ((uint32_t)(it / AT_KV_STAGES) & 1u) ^ 1u, abort_flag, prm.status)) break;
-        mbar_expect_tx(kv_full(s), AT_STAGE_BYTES);
-        tma_load_2d(sK(s), &map_k, kv_full(s), prm.k_col0 + h * AT_DH, b * prm.k_rows_per_seq + t * 128);
-        tma_load_2d(sVT(s), &map_vt, kv_full(s), t * 128, b * prm.d + h * AT_DH);
-        tma_load_2d(sVT(s) + 64 * 64 * 2, &map_vt, kv_full(s), t * 128 + 64, b * prm.d + h * AT_DH);
+        if (!mbar_wait_warp(kv_empty(s), ((uint32_t)(it / AT_KV_STAGES) & 1u) ^ 1u, abort_flag, prm.status)) break;
+        if (elect_one()) {
+          mbar_expect_tx(kv_full(s), AT_STAGE_BYTES);
+          tma_load_2d(sK(s), &map_k, kv_full(s), prm.k_col0 + h * AT_DH, b * prm.k_rows_per_seq + t * 128);
+          tma_load_2d(sVT(s), &map_vt, kv_full(s), t * 128, b * prm.d + h * AT_DH);
+          tma_load_2d(sVT(s) + 64 * 64 * 2, &map_vt, kv_full(s), t * 128 + 64, b * prm.d + h * AT_DH);
+        }
+        __syncwarp();
         issued = it + 1;
       }
-      if (*abort_flag) {   // do not leave while copies into this CTA's shared memory may be in flight
+      if (lane == 0 && *abort_flag) {   // do not leave while copies into this CTA's shared memory may be in flight
         long long t0 = clock64();
         while (!mbar_try(q_full, 0u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
         for (int t = issued > AT_KV_STAGES ? issued - AT_KV_STAGES : 0; t < issued; ++t) {
@@ -204,21 +209,24 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     }
     if (kv_split > 1) { __syncwarp(); cluster_sync_all(); }   // see the soft-max warps
   } else if (warp == 1) {
-    if (lane == 0 && my_kt > 0) {
+    if (my_kt > 0) {
       constexpr uint32_t idesc_s = make_idesc<128>();
       constexpr uint32_t idesc_pv = make_idesc<64>();
-      bool ok = mbar_wait(q_full, 0u, abort_flag, prm.status);
+      bool ok = mbar_wait_warp(q_full, 0u, abort_flag, prm.status);
       const uint64_t dq = make_smem_desc(sQ);
       // S(t) = Q K(t)^T into S buffer t & 1 (PIPE) or the one S buffer; t counts this CTA's iterations
       auto issue_s = [&](int t) -> bool {
         const int s = t % AT_KV_STAGES;
-        if (!mbar_wait(kv_full(s), (uint32_t)(t / AT_KV_STAGES) & 1u, abort_flag, prm.status)) return false;
+        if (!mbar_wait_warp(kv_full(s), (uint32_t)(t / AT_KV_STAGES) & 1u, abort_flag, prm.status)) return false;
         fence_after_sync();
         const uint64_t dk = make_smem_desc(sK(s));
         const uint32_t sc = PIPE ? (uint32_t)(t & 1) * 128u : 0u;
+        if (elect_one()) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) umma(tmem_base + sc, dq + 2u * k, dk + 2u * k, idesc_s, k > 0 ? 1u : 0u);
-        umma_commit(s_full(PIPE ? (t & 1) : 0));
+          for (int k = 0; k < 4; ++k) umma(tmem_base + sc, dq + 2u * k, dk + 2u * k, idesc_s, k > 0 ? 1u : 0u);
+          umma_commit(s_full(PIPE ? (t & 1) : 0));
+        }
+        __syncwarp();
         return true;
       };
       if (PIPE && ok) ok = issue_s(0);
@@ -232,21 +240,24 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
           ok = issue_s(t);
         }
         if (!ok) break;
-        ok = mbar_wait(p_ready(PIPE ? (t & 1) : 0), (uint32_t)(PIPE ? (t >> 1) : t) & 1u, abort_flag, prm.status);
+        ok = mbar_wait_warp(p_ready(PIPE ? (t & 1) : 0), (uint32_t)(PIPE ? (t >> 1) : t) & 1u, abort_flag, prm.status);
         if (!ok) break;
         fence_after_sync();
         // one accumulator per half of the key tile (keys 0..63 and keys 64..127 of the tile); both add up over the
         // CTA's tiles in TMEM
+        if (elect_one()) {
 #pragma unroll
-        for (int kb = 0; kb < 2; ++kb) {
-          const uint64_t dp = make_smem_desc(kb == 0 ? sK(s) : sP(t));
-          const uint64_t dv = make_smem_desc(sVT(s) + kb * (64 * 64 * 2));
+          for (int kb = 0; kb < 2; ++kb) {
+            const uint64_t dp = make_smem_desc(kb == 0 ? sK(s) : sP(t));
+            const uint64_t dv = make_smem_desc(sVT(s) + kb * (64 * 64 * 2));
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            umma(tmem_base + ACC_COL + (uint32_t)(kb * 64), dp + 2u * k, dv + 2u * k, idesc_pv, (t | k) ? 1u : 0u);
+            for (int k = 0; k < 4; ++k)
+              umma(tmem_base + ACC_COL + (uint32_t)(kb * 64), dp + 2u * k, dv + 2u * k, idesc_pv, (t | k) ? 1u : 0u);
+          }
+          umma_commit(pv_full(PIPE ? (t & 1) : 0));
+          umma_commit(kv_empty(s));
         }
-        umma_commit(pv_full(PIPE ? (t & 1) : 0));
-        umma_commit(kv_empty(s));
+        __syncwarp();
       }
     }
     if (kv_split > 1) { __syncwarp(); cluster_sync_all(); }
