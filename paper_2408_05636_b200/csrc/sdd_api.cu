@@ -253,7 +253,7 @@ static void fill_dims(const Net& P, const Net& Q, const sdd_params* p, int max_p
   if (lmax > D->tok_stride) lmax = D->tok_stride;
   D->lcap_max = (int)align_up((size_t)lmax, ROW_TILE);
   D->rows_q = (long long)p->batch * D->lcap_max;
-  const long long ver = (long long)p->batch * (p->gamma + 1), pre = (long long)p->batch * (max_prompt > 1 ? max_prompt - 1 : 0);
+  const long long ver = (long long)p->batch * (p->gamma + 1), pre = (long long)p->batch * (long long)align_up((size_t)(max_prompt - 1), ROW_TILE);
   D->rows_p = ver > pre ? ver : pre;
   D->max_prompt = max_prompt;
   D->esize = P.dtype == SDD_BF16 ? 2 : 4;
@@ -437,6 +437,16 @@ static int forward_causal(sdd_ctx* c, const Net& N, void* kv, const int* len, in
                     xf_lo, nullptr, nullptr, stats, stats_chunks));
   }
   return SDD_OK;
+}
+
+// Rows per sequence of a prefill of n tokens.  The fused QKV product stores K and V^T by TMA only where its 128-row tiles do
+// not straddle sequences; the rows added for that cost less than the element-wise stores of the other way up to about a
+// third (one sequence fills its last tile anyway), and rows past a prompt are computed like padding.
+template <typename T>
+static int prefill_rows(const sdd_ctx* c, const Net& N, int n) {
+  const int padded = (int)align_up((size_t)n, ROW_TILE);
+  if (!use_tc<T>(c, N) || padded > N.n_ctx || (long long)n * c->D.batch <= 64) return n;
+  return c->D.batch == 1 || 4 * padded <= 5 * n ? padded : n;
 }
 
 // target forward over rows_per_seq new tokens per sequence against the KV cache
@@ -644,6 +654,8 @@ int32_t sdd_create(const sdd_model* target, const sdd_model* drafter, const sdd_
   SDD_CUDA(prepare_attn());
   // the tensor-core attention multiplies masked probabilities (exact zeros) with whatever the V^T cache holds
   // past the valid positions, so that memory must be finite
+  // the activations likewise: padding rows have to be finite, and stay so in later generations
+  SDD_CUDA(cudaMemsetAsync(c->B.h, 0, (size_t)((uint8_t*)c->B.kv - (uint8_t*)c->B.h), c->st));
   SDD_CUDA(cudaMemsetAsync(c->B.kv, 0, (size_t)c->P.n_layer * params->batch * c->P.n_ctx * 2 * c->P.d * c->D.esize, c->st));
   s = load_prompts(c, prompt_ids, prompt_stride, prompt_len, max_prompt);
   if (s != SDD_OK) return s;
@@ -652,25 +664,24 @@ int32_t sdd_create(const sdd_model* target, const sdd_model* drafter, const sdd_
   return SDD_OK;
 }
 
-// start of a generation: zero the small state and the activations (padding rows must stay finite), load the prompts,
-// prefill the target's KV cache with x_{0:c-2}
+// start of a generation: zero the small state, load the prompts, prefill the target's KV cache with x_{0:c-2}
 static int load_prompts(sdd_ctx* c, const int32_t* prompt_ids, int32_t prompt_stride, const int32_t* prompt_len, int max_prompt) {
   const Buffers& B = c->B;
   const int batch = c->D.batch;
   const size_t state_bytes = (size_t)((uint8_t*)B.step_logits - (uint8_t*)B.rs);
   SDD_CUDA(cudaMemsetAsync(B.rs, 0, state_bytes, c->st));
-  const size_t act_bytes = (size_t)((uint8_t*)B.kv - (uint8_t*)B.h);
-  SDD_CUDA(cudaMemsetAsync(B.h, 0, act_bytes, c->st));
   SDD_CUDA(cudaMemcpy2DAsync(B.tokens, (size_t)c->D.tok_stride * 4, prompt_ids, (size_t)prompt_stride * 4,
                              (size_t)max_prompt * 4, batch, cudaMemcpyDeviceToDevice, c->st));
   SDD_CUDA(cudaMemcpyAsync(B.ctx_len, prompt_len, (size_t)batch * 4, cudaMemcpyHostToDevice, c->st));
+  SDD_CUDA(cudaEventRecord(c->ev[0], c->st));       // no round of this generation has used it yet
   c->D.max_prompt = max_prompt;
   int s;
-  if (c->P.dtype == SDD_BF16) s = forward_target<__nv_bfloat16>(c, TARGET_PREFILL, max_prompt - 1, false);
+  if (c->P.dtype == SDD_BF16)
+    s = forward_target<__nv_bfloat16>(c, TARGET_PREFILL, prefill_rows<__nv_bfloat16>(c, c->P, max_prompt - 1), false);
   else s = forward_target<float>(c, TARGET_PREFILL, max_prompt - 1, false);
   if (s != SDD_OK) return s;
-  // prompt_len is host memory owned by the caller: make sure the copy above has consumed it
-  SDD_CUDA(cudaStreamSynchronize(c->st));
+  // prompt_ids and prompt_len belong to the caller: the copies above have consumed them (the prefill goes on behind)
+  SDD_CUDA(cudaEventSynchronize(c->ev[0]));
   return SDD_OK;
 }
 
@@ -874,7 +885,7 @@ int32_t sdd_sps_attach(sdd_ctx* c, const sdd_model* ar_drafter, void* workspace,
 static int prefill_ar_drafter(sdd_ctx* c) {
   const Net& A = c->A;
   const Buffers& B = c->B;
-  const int rows = c->D.max_prompt - 1;
+  const int n = c->D.max_prompt - 1, rows = A.dtype == SDD_BF16 ? prefill_rows<__nv_bfloat16>(c, A, n) : n;
   int s = SDD_OK;
   if (A.dtype == SDD_BF16) {
     SDD_LAUNCH(c, CAT_GLUE, launch_embed_target<__nv_bfloat16>((const __nv_bfloat16*)A.wte, (const __nv_bfloat16*)A.wpe, B.tokens,

@@ -43,8 +43,9 @@ constexpr int BK = 64;           // 64 bf16 = 128 bytes = one swizzle row
 constexpr int UMMA_K = 16;
 constexpr int THREADS = 192;     // warp 0: TMA producer, warp 1: MMA issuer + TMEM owner, warps 2-5: epilogue
 
-// tensor maps of the epilogue's TMA stores: the output matrix and (fused QKV of the drafter) the transposed V tensor
-struct alignas(64) OutMaps { CUtensorMap out, vt; };
+// tensor maps of the epilogue's TMA stores: the output matrix; the K cache and the transposed V tensor of a fused QKV
+// product; the second half of a hi/lo output pair takes the place of `vt`
+struct alignas(64) OutMaps { CUtensorMap out, vt, k; };
 
 // one stage = A tile + B tile (+ the lo tile of the activation operand: the A side unless SWAP)
 template <int BN, bool SWAP, bool HILO>
@@ -171,48 +172,126 @@ __device__ __forceinline__ void epilogue_tma(uint32_t tmem_acc, int m0, int n0, 
   }
 }
 
-// V tiles of the drafter's fused-QKV GEMM: the tile is written transposed ([feature][position]) into the staging
-// buffers -- 64 features x 128 positions per buffer, as two 128-byte-swizzled boxes of 64 positions -- and leaves
-// through two TMA tile stores per buffer.  The 128 rows of the tile are 128 consecutive positions of one sequence.
-// vt_row0: row of the tile's first feature in the V^T tensor; pos0: position of the tile's first row.
+// Fused QKV product over token rows that are consecutive positions of one sequence (128-row tiles never straddle
+// sequences): every 64 columns belong to Q, K or V (d is a multiple of 64) and leave through one staging buffer.  Q, and
+// K where it stays next to Q, go to the output rows, K with a cache to the cache's rows; V is written transposed
+// ([feature][position]: 64 features x 128 positions per buffer, as two 128-byte-swizzled boxes of 64 positions) and leaves
+// through two tile stores.  Rows past the end of a prompt are stored like the others: their positions are written again
+// before anything reads them.
 template <int BN>
-__device__ __forceinline__ void epilogue_vt(uint32_t tmem_acc, int q, int lane, const float* bias_s,
-                                            const CUtensorMap* map_vt, uint8_t* stage_generic, uint32_t stage_u32,
-                                            int& n_store, int vt_row0, int pos0,
-                                            const EpiGroup eg = whole_tile_group<BN>()) {
+__device__ __forceinline__ void epilogue_qkv(uint32_t tmem_acc, int m0, int n0, int q, int lane, const float* bias_s,
+                                             const OutMaps& maps, const QkvDst& qd, uint8_t* stage_generic,
+                                             uint32_t stage_u32, int& n_store, const EpiGroup eg = whole_tile_group<BN>()) {
   const int rl = q * 32 + lane;               // row inside the tile = position offset
+  const int sw = rl & 7;
   const bool is_issuer = (int)threadIdx.x == eg.first_tid;
   const int pl = rl & 63;
   const uint32_t box_off = (uint32_t)(rl >> 6) * (64 * 128);       // positions 64..127 fill the second box
   const uint32_t in_row = (uint32_t)(pl & 7) * 2u;
   const uint32_t pchunk = (uint32_t)(pl >> 3);
+  const int sb = m0 / qd.rows_per_seq, pos0 = m0 - sb * qd.rows_per_seq;
 #pragma unroll 1
   for (int cc = eg.c_begin; cc < eg.c_end; ++cc) {
+    const int c0 = n0 + (cc & ~1) * 32;       // first column of the buffer
+    if (c0 >= 3 * qd.d) break;
+    const bool is_v = c0 >= 2 * qd.d;
     uint32_t v[32];
     tmem_ld32(tmem_acc + ((uint32_t)(q * 32) << 16) + (uint32_t)(cc * 32), v);
     const int buf = eg.nbuf == 1 ? 0 : ((cc >> 1) & 1);
-    const bool first_of_buf = (cc & 1) == 0;
-    const bool last_of_buf = (cc & 1) == 1 || cc == eg.c_end - 1;
-    if (first_of_buf) {
+    if ((cc & 1) == 0) {
       // the stores that last used this buffer have read it
       if (is_issuer && n_store >= eg.nbuf) { if (eg.nbuf == 1) tma_wait_group_read<0>(); else tma_wait_group_read<1>(); }
       named_bar_sync(eg.bar_id, 128);
     }
-    uint8_t* bp = stage_generic + buf * (128 * 128) + box_off;
+    uint8_t* bp = stage_generic + buf * (128 * 128);
+    if (is_v) {
+      bp += box_off;
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const int jj = (cc & 1) * 32 + j;        // feature row inside the buffer
-      const float x = __uint_as_float(v[j]) + bias_s[cc * 32 + j];
-      *reinterpret_cast<__nv_bfloat16*>(bp + jj * 128 + ((pchunk ^ (uint32_t)(jj & 7)) << 4) + in_row) = __float2bfloat16_rn(x);
+      for (int j = 0; j < 32; ++j) {
+        const int jj = (cc & 1) * 32 + j;      // feature row inside the buffer
+        const float x = __uint_as_float(v[j]) + bias_s[cc * 32 + j];
+        *reinterpret_cast<__nv_bfloat16*>(bp + jj * 128 + ((pchunk ^ (uint32_t)(jj & 7)) << 4) + in_row) = __float2bfloat16_rn(x);
+      }
+    } else {
+      uint8_t* row = bp + rl * 128;
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        uint32_t pk[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int j0 = g * 8 + 2 * e;
+          __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(v[j0]) + bias_s[cc * 32 + j0],
+                                                    __uint_as_float(v[j0 + 1]) + bias_s[cc * 32 + j0 + 1]);
+          pk[e] = *reinterpret_cast<uint32_t*>(&h2);
+        }
+        *reinterpret_cast<uint4*>(row + ((((cc & 1) * 4 + g) ^ sw) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+      }
     }
-    if (last_of_buf) {
+    if ((cc & 1) == 1) {
       fence_async_smem();
       named_bar_sync(eg.bar_id, 128);
       if (is_issuer) {
         const uint32_t src = stage_u32 + buf * (128 * 128);
-        const int y = vt_row0 + (cc & ~1) * 32;
-        tma_store_2d(map_vt, src, pos0, y);
-        tma_store_2d(map_vt, src + 64 * 128, pos0 + 64, y);
+        if (is_v) {
+          const int y = sb * qd.d + c0 - 2 * qd.d;
+          tma_store_2d(&maps.vt, src, pos0, y);
+          tma_store_2d(&maps.vt, src + 64 * 128, pos0 + 64, y);
+        } else if (c0 >= qd.d && qd.k_dst != nullptr) {
+          tma_store_2d(&maps.k, src, c0 - qd.d, sb * qd.k_seq_rows + pos0);
+        } else {
+          tma_store_2d(&maps.out, src, c0, m0);
+        }
+        tma_commit_group();
+      }
+      ++n_store;
+    }
+  }
+}
+
+// bf16 output as a hi/lo pair, hi = bf16(x) to maps.out and lo = bf16(x - hi) to maps.vt: 64 columns at a time, the two
+// halves one after the other through the group's staging buffers (the accumulator and the activation are evaluated twice,
+// which costs less than another 16 KB of shared memory taken from the operand ring).
+template <int BN>
+__device__ __forceinline__ void epilogue_pair_out(uint32_t tmem_acc, int m0, int n0, int q, int lane, int epi, const float* bias_s,
+                                                  const OutMaps& maps, uint8_t* stage_generic, uint32_t stage_u32, int& n_store,
+                                                  const EpiGroup eg = whole_tile_group<BN>()) {
+  const int rl = q * 32 + lane, sw = rl & 7;
+  const bool is_issuer = (int)threadIdx.x == eg.first_tid;
+#pragma unroll 1
+  for (int it = eg.c_begin; it < 2 * eg.c_end - eg.c_begin; ++it) {
+    // per 64 columns: chunk 0 and 1 of hi, chunk 0 and 1 of lo
+    const int rel = it - eg.c_begin, cc = eg.c_begin + (rel >> 2) * 2 + (rel & 1);
+    const bool lo = (rel & 2) != 0;
+    uint32_t v[32];
+    tmem_ld32(tmem_acc + ((uint32_t)(q * 32) << 16) + (uint32_t)(cc * 32), v);
+    const int buf = eg.nbuf == 1 ? 0 : (lo ? 1 : 0);
+    if ((cc & 1) == 0) {
+      if (is_issuer && n_store >= eg.nbuf) { if (eg.nbuf == 1) tma_wait_group_read<0>(); else tma_wait_group_read<1>(); }
+      named_bar_sync(eg.bar_id, 128);
+    }
+    uint8_t* row = stage_generic + buf * (128 * 128) + rl * 128;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      uint32_t pk[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int j0 = g * 8 + 2 * e;
+        float x0 = __uint_as_float(v[j0]) + bias_s[cc * 32 + j0], x1 = __uint_as_float(v[j0 + 1]) + bias_s[cc * 32 + j0 + 1];
+        if (epi == EPI_GELU) { x0 = gelu_tanh_fast(x0); x1 = gelu_tanh_fast(x1); }
+        __nv_bfloat162 h2 = __floats2bfloat162_rn(x0, x1);
+        if (lo) {
+          const uint32_t hb = *reinterpret_cast<uint32_t*>(&h2);
+          h2 = __floats2bfloat162_rn(x0 - __uint_as_float(hb << 16), x1 - __uint_as_float(hb & 0xffff0000u));
+        }
+        pk[e] = *reinterpret_cast<uint32_t*>(&h2);
+      }
+      *reinterpret_cast<uint4*>(row + ((((cc & 1) * 4 + g) ^ sw) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    }
+    if ((cc & 1) == 1) {
+      fence_async_smem();
+      named_bar_sync(eg.bar_id, 128);
+      if (is_issuer) {
+        tma_store_2d(lo ? &maps.vt : &maps.out, stage_u32 + buf * (128 * 128), n0 + (cc & ~1) * 32, m0);
         tma_commit_group();
       }
       ++n_store;
@@ -581,7 +660,15 @@ __device__ __forceinline__ void epilogue_head_normal(uint32_t tmem_acc, int m0, 
 template <int BN, bool SWAP>
 constexpr int one_tile_threads() { return (!SWAP && BN >= 128) ? 320 : THREADS; }
 
-template <int BN, bool SWAP, bool HILO, bool DEEP>
+// OUT: how the tile leaves.  One kernel per way: a CTA runs through its epilogue once, and code for the other ways only
+// lengthens its instruction fetches (all of them in one kernel: XL batch-1 round 21.35 -> 21.59 ms).
+enum OutWay : int {
+  OUT_ANY = 0,    // by hand or (SWAP, residual stream) by add-reduce: every epilogue, any alignment
+  OUT_ROWS = 1,   // row-major tiles by TMA: bf16 stores, add-reduce into the residual stream
+  OUT_QKV = 2,    // fused QKV over whole tiles of positions, by TMA
+  OUT_PAIR = 3    // a hi/lo pair of bf16 tiles by TMA
+};
+template <int BN, bool SWAP, bool HILO, bool DEEP, int OUT>
 __global__ void __launch_bounds__(one_tile_threads<BN, SWAP>())
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_lo, const __grid_constant__ OutMaps maps_out, int tma_out,
@@ -731,34 +818,27 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const EpiGroup eg = TWO ? EpiGroup{grp * (BN / 64), (grp + 1) * (BN / 64), 2, 2 + grp, 64 + grp * 128} : whole_tile_group<BN>();
     uint8_t* stage_g = generic_base + grp * (2 * 128 * 128);
     const uint32_t stage_u = base + grp * (2 * 128 * 128);
-    // every lane waits; the outcome is made warp-uniform because tcgen05.ld is a warp-wide instruction
-    // (and uniform over the four warps of a group, which meet at named barriers in the TMA-store path)
-    float* bias_s = reinterpret_cast<float*>(generic_base + STAGES * STAGE_BYTES + 256);
-    // tma_out == 2 (fused QKV): only tiles that lie wholly in the columns kept in place (Q, and K without a cache)
-    // are plain row-major stores; the others scatter into the K cache / V^T and take the manual path
-    // tma_out == 3: also the tiles that lie wholly in V leave by TMA, transposed (drafter; 128-row tiles never
-    // straddle sequences there)
-    const bool use_tma = !SWAP && (tma_out == 1 || (tma_out >= 2 && n0 + BN <= (qd.k_dst != nullptr ? qd.d : 2 * qd.d)));
-    const bool vt_tma = !SWAP && tma_out == 3 && n0 >= 2 * qd.d && n0 + BN <= rows_b;
-    if (use_tma || vt_tma) stage_bias(bias_s, bias, n0, rows_b, eg);     // while the main loop runs
+    // every lane waits; the outcome is made uniform over the four warps of a group (tcgen05.ld is a warp-wide instruction,
+    // and they meet at named barriers in the TMA-store path)
+    [[maybe_unused]] float* bias_s = reinterpret_cast<float*>(generic_base + STAGES * STAGE_BYTES + 256);
+    if constexpr (OUT != OUT_ANY) stage_bias(bias_s, bias, n0, rows_b, eg);     // while the main loop runs
     const bool ready = named_bar_and(TWO ? 4 + grp : 1, 128, mbar_wait(tmem_full_bar, 0u, abort_flag, status));
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (ready && use_tma) {
+    if (ready) {
       int n_store = 0;
-      epilogue_tma<BN>(tmem_base, m0, n0, q, lane, epi == EPI_QKV ? (int)EPI_STORE : epi, bias_s, &maps_out.out, stage_g, stage_u,
-                       n_store, eg);
-      if ((int)threadIdx.x == eg.first_tid) tma_wait_group_read<0>();      // shared memory stays valid until the copies have read it
-    } else if (ready && vt_tma) {
-      int n_store = 0;
-      const int sb = m0 / qd.rows_per_seq;
-      epilogue_vt<BN>(tmem_base, q, lane, bias_s, &maps_out.vt, stage_g, stage_u, n_store, sb * qd.d + (n0 - 2 * qd.d),
-                      m0 - sb * qd.rows_per_seq, eg);
-      if ((int)threadIdx.x == eg.first_tid) tma_wait_group_read<0>();
-    } else if (ready && SWAP && tma_out == 4) {
-      if constexpr (SWAP) epilogue_swap_reduce<BN>(tmem_base, m0, n0, q, lane, rows_a, bias, &maps_out.out, generic_base, base);
-    } else if (ready) {
-      epilogue_manual<BN, SWAP, SWAP>(tmem_base, m0, n0, q, lane, rows_a, rows_b, epi, bias, out, out_lo, ldc, split, qd, eg.c_begin,
-                                      eg.c_end);
+      if constexpr (OUT == OUT_ROWS) {
+        epilogue_tma<BN>(tmem_base, m0, n0, q, lane, epi, bias_s, &maps_out.out, stage_g, stage_u, n_store, eg);
+      } else if constexpr (OUT == OUT_QKV) {
+        epilogue_qkv<BN>(tmem_base, m0, n0, q, lane, bias_s, maps_out, qd, stage_g, stage_u, n_store, eg);
+      } else if constexpr (OUT == OUT_PAIR) {
+        epilogue_pair_out<BN>(tmem_base, m0, n0, q, lane, epi, bias_s, maps_out, stage_g, stage_u, n_store, eg);
+      } else if (SWAP && tma_out == 4) {
+        if constexpr (SWAP) epilogue_swap_reduce<BN>(tmem_base, m0, n0, q, lane, rows_a, bias, &maps_out.out, generic_base, base);
+      } else {
+        epilogue_manual<BN, SWAP, SWAP>(tmem_base, m0, n0, q, lane, rows_a, rows_b, epi, bias, out, out_lo, ldc, split, qd, eg.c_begin,
+                                        eg.c_end);
+      }
+      if (OUT != OUT_ANY && (int)threadIdx.x == eg.first_tid) tma_wait_group_read<0>();   // shared memory stays valid until the copies have read it
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -933,9 +1013,8 @@ gemm_tc_persist_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
       const int m0 = (n_fastest ? tile / tiles_n : tile % tiles_m) * BM;
       const int n0 = (n_fastest ? tile % tiles_n : tile / tiles_m) * BN;
       float* bias_s = reinterpret_cast<float*>(generic_base + BAR_OFF + 512) + buf * BN;
-      const bool use_tma = !SWAP && (tma_out == 1 || (tma_out >= 2 && n0 + BN <= (qd.k_dst != nullptr ? qd.d : 2 * qd.d)));
-      const bool vt_tma = !SWAP && tma_out == 3 && n0 >= 2 * qd.d && n0 + BN <= rows_b;
-      if (use_tma || vt_tma) stage_bias<BN>(bias_s, bias, n0, rows_b);  // while the tile's main loop runs
+      const bool use_tma = !SWAP && (tma_out == 1 || (tma_out == 2 && n0 + BN <= qd.d));
+      if (!SWAP && (use_tma || tma_out == 3 || tma_out == 5)) stage_bias<BN>(bias_s, bias, n0, rows_b);  // while the tile's main loop runs
       const bool ready = named_bar_and(1, 128, mbar_wait(tfull_bar(buf), (uint32_t)(i >> 1) & 1u, abort_flag, status));
       if (!ready) break;
       fence_after_sync();
@@ -950,9 +1029,13 @@ gemm_tc_persist_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
       else if (use_tma)
         epilogue_tma<BN>(acc, m0, n0, q, lane, epi == EPI_QKV ? (int)EPI_STORE : epi, bias_s, &maps_out.out,
                          generic_base + STAGING_OFF, base + STAGING_OFF, n_store);
-      else if (vt_tma)
-        epilogue_vt<BN>(acc, q, lane, bias_s, &maps_out.vt, generic_base + STAGING_OFF, base + STAGING_OFF, n_store,
-                        (m0 / qd.rows_per_seq) * qd.d + (n0 - 2 * qd.d), m0 % qd.rows_per_seq);
+      else if (!HILO && tma_out == 3) {
+        if constexpr (!HILO)
+          epilogue_qkv<BN>(acc, m0, n0, q, lane, bias_s, maps_out, qd, generic_base + STAGING_OFF, base + STAGING_OFF, n_store);
+      } else if (HILO && tma_out == 5) {
+        if constexpr (HILO)
+          epilogue_pair_out<BN>(acc, m0, n0, q, lane, epi, bias_s, maps_out, generic_base + STAGING_OFF, base + STAGING_OFF, n_store);
+      }
       else
         epilogue_manual<BN, false>(acc, m0, n0, q, lane, rows_a, rows_b, epi, bias, out, out_lo, ldc, false, qd);
       // this thread's reads of the accumulator are complete (tcgen05.wait::ld inside tmem_ld32): hand it back
@@ -988,21 +1071,23 @@ gemm_tc_persist_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
 // (columns 0..127 and 128..255, one staging buffer each), because the main loop of a tile is a third shorter here.  The CTAs meet at a cluster
 // barrier before TMEM is freed, so that neither leaves while the other may still touch its shared memory.
 // ---------------------------------------------------------------------------------------------
-constexpr int PAIR_STAGE_BYTES = BM * BK * 2 + 128 * BK * 2;     // A tile + half of the 256-wide B tile: 32 KB
-constexpr int PAIR_STAGES = 6;
-constexpr int PAIR_STAGING_OFF = PAIR_STAGES * PAIR_STAGE_BYTES;
+// a stage: A tile + half of the 256-wide B tile, 32 KB, + the lo tile of the activations, 48 KB: 192 KB of ring either way
+template <bool HILO> constexpr int pair_stage_bytes() { return (HILO ? 3 : 2) * BM * BK * 2; }
+template <bool HILO> constexpr int pair_stages() { return HILO ? 4 : 6; }
+constexpr int PAIR_STAGING_OFF = 192 * 1024;
 constexpr int PAIR_BAR_OFF = PAIR_STAGING_OFF + 2 * 128 * 128;
 constexpr int PAIR_SMEM = PAIR_BAR_OFF + 512 + 1024 + 1024;       // barriers, one tile's bias, alignment slack
 
 constexpr int PAIR_THREADS = 320;   // warp 0: TMA, warp 1: MMA (leader) + TMEM owner, warps 2-5 and 6-9: two epilogue groups
 
+template <bool HILO>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PAIR_THREADS)
 gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                    const __grid_constant__ OutMaps maps_out, int tma_out, int rows_a, int rows_b, int K, int epi,
+                    const __grid_constant__ CUtensorMap map_lo, const __grid_constant__ OutMaps maps_out, int tma_out, int rows_a, int rows_b, int K, int epi,
                     const float* __restrict__ bias, void* __restrict__ out, int ldc, int* status, const QkvDst qd,
                     const int* __restrict__ skip, int tiles_m2, int tiles_n, int n_fastest) {
   constexpr int BN = 256;
-  constexpr int STAGES = PAIR_STAGES;
+  constexpr int STAGES = pair_stages<HILO>(), PAIR_STAGE_BYTES = pair_stage_bytes<HILO>();
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* generic_base = smem_raw + (base - smem_u32(smem_raw));
@@ -1056,6 +1141,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           const uint32_t sa = base + s * PAIR_STAGE_BYTES;
           tma_load_2d_pair(sa, &map_a, lf, kb * BK, m0);
           tma_load_2d_pair(sa + BM * BK * 2, &map_b, lf, kb * BK, n0);
+          if (HILO) tma_load_2d_pair(sa + 2 * BM * BK * 2, &map_lo, lf, kb * BK, m0);
         }
         __syncwarp();
       }
@@ -1091,6 +1177,12 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 #pragma unroll
             for (int k = 0; k < BK / UMMA_K; ++k)
               umma_pair(acc, da + (uint64_t)(k * UMMA_K * 2 / 16), db + (uint64_t)(k * UMMA_K * 2 / 16), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+            if (HILO) {
+              const uint64_t dl = make_smem_desc(sa + 2 * BM * BK * 2);
+#pragma unroll
+              for (int k = 0; k < BK / UMMA_K; ++k)
+                umma_pair(acc, dl + (uint64_t)(k * UMMA_K * 2 / 16), db + (uint64_t)(k * UMMA_K * 2 / 16), idesc, 1u);
+            }
             umma_commit_pair(empty_bar(s));                       // frees the stage in this CTA ...
             umma_commit_pair(map_to_cta(empty_bar(s), peer));     // ... and in the peer
             if (kb == num_kb - 1) umma_commit_pair(tfull_bar(buf));
@@ -1113,9 +1205,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       const int m0 = (n_fastest ? tile / tiles_n : tile % tiles_m2) * (2 * BM) + (int)rank * BM;
       const int n0 = (n_fastest ? tile % tiles_n : tile / tiles_m2) * BN;
       float* bias_s = reinterpret_cast<float*>(generic_base + PAIR_BAR_OFF + 512);   // reused: the same threads read it last
-      const bool use_tma = tma_out == 1 || (tma_out >= 2 && n0 + BN <= (qd.k_dst != nullptr ? qd.d : 2 * qd.d));
-      const bool vt_tma = tma_out == 3 && n0 >= 2 * qd.d && n0 + BN <= rows_b;
-      if (use_tma || vt_tma) stage_bias(bias_s, bias, n0, rows_b, eg);  // while the tile's main loop runs
+      stage_bias(bias_s, bias, n0, rows_b, eg);        // while the tile's main loop runs
       const bool mine = mbar_wait_cluster(tfull_bar(buf), (uint32_t)(i >> 1) & 1u, abort_flag, status);
       // the leader forwards "accumulator complete" to the peer's epilogue warps
       if (leader && threadIdx.x == 64 && mine) mbar_arrive_remote_relaxed(map_to_cta(tfull_bar(buf), peer));
@@ -1123,15 +1213,18 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       if (!ready) break;
       fence_after_sync();
       const uint32_t acc = tmem_base + (uint32_t)(buf * BN);
-      if (use_tma)
-        epilogue_tma<BN>(acc, m0, n0, q, lane, epi == EPI_QKV ? (int)EPI_STORE : epi, bias_s, &maps_out.out, stage_g, stage_u,
-                         n_store, eg);
-      else if (vt_tma)
-        epilogue_vt<BN>(acc, q, lane, bias_s, &maps_out.vt, stage_g, stage_u, n_store,
-                        (m0 / qd.rows_per_seq) * qd.d + (n0 - 2 * qd.d), m0 % qd.rows_per_seq, eg);
-      else
-        epilogue_manual<BN, false>(acc, m0, n0, q, lane, rows_a, rows_b, epi, bias, out, nullptr, ldc, false, qd, eg.c_begin,
-                                   eg.c_end);
+      if (m0 >= rows_a) {
+        // the lower half of the last row of tiles may lie past the matrix
+      } else if (tma_out == 1) {
+        epilogue_tma<BN>(acc, m0, n0, q, lane, epi, bias_s, &maps_out.out, stage_g, stage_u, n_store, eg);
+      } else if (tma_out == 3) {
+        if constexpr (!HILO) epilogue_qkv<BN>(acc, m0, n0, q, lane, bias_s, maps_out, qd, stage_g, stage_u, n_store, eg);
+      } else if (tma_out == 5) {
+        if constexpr (HILO) epilogue_pair_out<BN>(acc, m0, n0, q, lane, epi, bias_s, maps_out, stage_g, stage_u, n_store, eg);
+      } else {
+        if constexpr (!HILO)
+          epilogue_manual<BN, false>(acc, m0, n0, q, lane, rows_a, rows_b, epi, bias, out, nullptr, ldc, false, qd, eg.c_begin, eg.c_end);
+      }
       // the warp's reads of the accumulator are complete (tcgen05.wait::ld inside tmem_ld32): hand it back, one arrive
       // per warp
       fence_before_sync();
@@ -1198,26 +1291,19 @@ __global__ void __launch_bounds__(THREADS) wait_timeout_probe_kernel(long long l
 // ---------------------------------------------------------------------------------------------
 // host side: tensor maps (cached per pointer / shape / box) and launch
 // ---------------------------------------------------------------------------------------------
-template <int BN, bool SWAP, bool HILO, bool DEEP>
-static cudaError_t launch_cfg2(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& ml, const OutMaps& mo,
-                              int tma_out, int rows_a, int rows_b, int K, int epi, const float* bias, void* out, void* out_lo,
-                              int ldc, int* status, cudaStream_t st, const QkvDst& qd, int splits, const int* skip) {
-  dim3 grid((rows_b + BN - 1) / BN, (rows_a + BM - 1) / BM, splits);
-  launch_k(gemm_tc_kernel<BN, SWAP, HILO, DEEP>, grid, dim3(one_tile_threads<BN, SWAP>()), smem_bytes<BN, SWAP, HILO, DEEP>(), st, ma, mb, ml, mo, tma_out,
-           rows_a, rows_b, K, epi, bias, out, out_lo, ldc, status, qd, skip);
-  return cudaGetLastError();
-}
-template <int BN, bool SWAP, bool HILO>
+template <int BN, bool SWAP, bool HILO, int OUT>
 static cudaError_t launch_cfg(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& ml, const OutMaps& mo,
                               int tma_out, int rows_a, int rows_b, int K, int epi, const float* bias, void* out, void* out_lo,
                               int ldc, int* status, cudaStream_t st, const QkvDst& qd, int splits, const int* skip) {
+  const dim3 grid((rows_b + BN - 1) / BN, (rows_a + BM - 1) / BM, splits), block(one_tile_threads<BN, SWAP>());
   // more than two waves of CTAs: shallow rings, two CTAs per SM (needs 2 x BN TMEM columns <= 512: always true)
-  const long long ctas = (long long)((rows_b + BN - 1) / BN) * ((rows_a + BM - 1) / BM) * splits;
-  if (ctas > 2 * 148)
-    return launch_cfg2<BN, SWAP, HILO, false>(ma, mb, ml, mo, tma_out, rows_a, rows_b, K, epi, bias, out, out_lo, ldc, status,
-                                              st, qd, splits, skip);
-  return launch_cfg2<BN, SWAP, HILO, true>(ma, mb, ml, mo, tma_out, rows_a, rows_b, K, epi, bias, out, out_lo, ldc, status, st,
-                                           qd, splits, skip);
+  if ((long long)grid.x * grid.y * grid.z > 2 * 148)
+    launch_k(gemm_tc_kernel<BN, SWAP, HILO, false, OUT>, grid, block, smem_bytes<BN, SWAP, HILO, false>(), st, ma, mb, ml, mo, tma_out,
+             rows_a, rows_b, K, epi, bias, out, out_lo, ldc, status, qd, skip);
+  else
+    launch_k(gemm_tc_kernel<BN, SWAP, HILO, true, OUT>, grid, block, smem_bytes<BN, SWAP, HILO, true>(), st, ma, mb, ml, mo, tma_out,
+             rows_a, rows_b, K, epi, bias, out, out_lo, ldc, status, qd, skip);
+  return cudaGetLastError();
 }
 template <int BN, bool HILO>
 static cudaError_t launch_persist(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& ml, const OutMaps& mo,
@@ -1259,20 +1345,37 @@ static cudaError_t launch_hl(bool hilo, const CUtensorMap& ma, const CUtensorMap
                              const OutMaps& mo, int tma_out, int rows_a, int rows_b, int K, int epi, const float* bias,
                              void* out, void* out_lo, int ldc, int* status, cudaStream_t st, const QkvDst& qd, int splits,
                              const int* skip) {
-  if (hilo)
-    return launch_cfg<BN, SWAP, true>(ma, mb, ml, mo, tma_out, rows_a, rows_b, K, epi, bias, out, out_lo, ldc, status, st, qd, splits, skip);
-  return launch_cfg<BN, SWAP, false>(ma, mb, ml, mo, tma_out, rows_a, rows_b, K, epi, bias, out, out_lo, ldc, status, st, qd, splits, skip);
+#define SDD_ONE(HILO_, OUT_) \
+  return launch_cfg<BN, SWAP, HILO_, OUT_>(ma, mb, ml, mo, tma_out, rows_a, rows_b, K, epi, bias, out, out_lo, ldc, status, st, qd, splits, skip)
+  if constexpr (!SWAP && BN >= 64) {
+    if (tma_out == 5) SDD_ONE(true, OUT_PAIR);
+    if (tma_out == 3 && !hilo) SDD_ONE(false, OUT_QKV);
+    if (tma_out == 1) { if (hilo) SDD_ONE(true, OUT_ROWS); SDD_ONE(false, OUT_ROWS); }
+  } else if constexpr (!SWAP) {
+    if (tma_out == 1) { if (hilo) SDD_ONE(true, OUT_ROWS); SDD_ONE(false, OUT_ROWS); }
+  }
+  if (hilo) SDD_ONE(true, OUT_ANY);
+  SDD_ONE(false, OUT_ANY);
+#undef SDD_ONE
 }
 
+template <int BN, bool SWAP, bool HILO, int OUT>
+static cudaError_t prepare_out() {
+  cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN, SWAP, HILO, true, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       smem_bytes<BN, SWAP, HILO, true>());
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(gemm_tc_kernel<BN, SWAP, HILO, false, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              smem_bytes<BN, SWAP, HILO, false>());
+}
 template <int BN, bool SWAP>
 static cudaError_t prepare_one() {
   cudaError_t e;
-#define SDD_PREP(HILO, DEEP)                                                                                      \
-  e = cudaFuncSetAttribute(gemm_tc_kernel<BN, SWAP, HILO, DEEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                           smem_bytes<BN, SWAP, HILO, DEEP>());                                                \
-  if (e != cudaSuccess) return e;
-  SDD_PREP(false, true) SDD_PREP(false, false) SDD_PREP(true, true) SDD_PREP(true, false)
-#undef SDD_PREP
+  if ((e = prepare_out<BN, SWAP, false, OUT_ANY>()) != cudaSuccess || (e = prepare_out<BN, SWAP, true, OUT_ANY>()) != cudaSuccess) return e;
+  if constexpr (!SWAP) {
+    if ((e = prepare_out<BN, SWAP, false, OUT_ROWS>()) != cudaSuccess || (e = prepare_out<BN, SWAP, true, OUT_ROWS>()) != cudaSuccess) return e;
+    if constexpr (BN >= 64)
+      if ((e = prepare_out<BN, SWAP, false, OUT_QKV>()) != cudaSuccess || (e = prepare_out<BN, SWAP, true, OUT_PAIR>()) != cudaSuccess) return e;
+  }
   return cudaSuccess;
 }
 
@@ -1303,7 +1406,8 @@ cudaError_t tc_prepare_gemm() {
                                 persist_smem_bytes<BN_, HL_, true>())) != cudaSuccess) return e;
   SDD_PREP_PS(32, false) SDD_PREP_PS(32, true) SDD_PREP_PS(64, false) SDD_PREP_PS(64, true)
 #undef SDD_PREP_PS
-  return cudaFuncSetAttribute(gemm_tc_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PAIR_SMEM);
+  if ((e = cudaFuncSetAttribute(gemm_tc_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PAIR_SMEM)) != cudaSuccess) return e;
+  return cudaFuncSetAttribute(gemm_tc_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PAIR_SMEM);
 }
 
 static PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
@@ -1398,7 +1502,7 @@ cudaError_t launch_gemm_tc(const __nv_bfloat16* A, long long a_cap, const __nv_b
     ml = mb;
     if (hilo && (e = get_tensor_map(A_lo, a_cap, K, K, bn, BK, &ml)) != cudaSuccess) return e;
     OutMaps none;
-    none.out = ma; none.vt = ma;
+    none.out = ma; none.vt = ma; none.k = ma;
     // fp32 residual stream with 16-byte-aligned rows: the tile leaves as TMA add-reduces (see epilogue_swap_reduce)
     int swap_tma = 0;
     if (epi == EPI_RESIDUAL && (ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0) {
@@ -1449,22 +1553,30 @@ cudaError_t launch_gemm_tc(const __nv_bfloat16* A, long long a_cap, const __nv_b
   if (hilo && (e = get_tensor_map(A_lo, a_cap, K, K, BM, BK, &ml)) != cudaSuccess) return e;
   // output through TMA where the layout allows 16-byte-aligned rows (see the kernel's epilogue)
   OutMaps mo;
-  mo.out = ma; mo.vt = ma;
+  mo.out = ma; mo.vt = ma; mo.k = ma;
   int tma_out = 0;
   if (epi == EPI_RESIDUAL && (ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0) {
     if ((e = get_tensor_map(out, M, N, ldc, BM, 32, &mo.out, 4)) != cudaSuccess) return e;
     tma_out = 1;
-  } else if ((epi == EPI_STORE || epi == EPI_GELU || epi == EPI_QKV) && out_lo == nullptr && bn >= 64 && (ldc & 7) == 0 &&
-             (reinterpret_cast<uintptr_t>(out) & 15u) == 0) {
+  } else if ((epi == EPI_STORE || epi == EPI_GELU || epi == EPI_QKV) && (out_lo == nullptr || hilo) && bn >= 64 && (ldc & 7) == 0 &&
+             ((reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(out_lo)) & 15u) == 0) {
     if ((e = get_tensor_map(out, M, N, ldc, BM, 64, &mo.out, 2)) != cudaSuccess) return e;
-    tma_out = epi == EPI_QKV ? 2 : 1;   // fused QKV: per tile, see the kernel
-    // drafter (every row of a tile is a position of one sequence, all of them stored): V tiles by TMA too
-    if (epi == EPI_QKV && qd.mode == 0 && qd.vt_dst != nullptr && (M % BM) == 0 && (qd.rows_per_seq % BM) == 0 &&
-        (qd.vt_ld & 7) == 0 && (reinterpret_cast<uintptr_t>(qd.vt_dst) & 15u) == 0 && qd.rows_per_seq <= qd.vt_ld) {
-      if ((e = get_tensor_map(qd.vt_dst, (long long)(M / qd.rows_per_seq) * qd.d, qd.vt_ld, qd.vt_ld, 64, 64, &mo.vt, 2)) !=
-          cudaSuccess)
-        return e;
-      tma_out = 3;
+    tma_out = 1;
+    if (out_lo != nullptr) {
+      if ((e = get_tensor_map(out_lo, M, N, ldc, BM, 64, &mo.vt, 2)) != cudaSuccess) return e;
+      tma_out = 5;
+    } else if (epi == EPI_QKV) {
+      tma_out = 2;
+      // drafter, prefill: every row of a tile is a position of one sequence
+      const int seqs = qd.rows_per_seq > 0 ? M / qd.rows_per_seq : 0;
+      if (qd.mode != 1 && qd.vt_dst != nullptr && (M % BM) == 0 && (qd.rows_per_seq % BM) == 0 && (qd.vt_ld & 7) == 0 &&
+          (reinterpret_cast<uintptr_t>(qd.vt_dst) & 15u) == 0 && qd.rows_per_seq <= qd.vt_ld &&
+          (qd.k_dst == nullptr || ((reinterpret_cast<uintptr_t>(qd.k_dst) & 15u) == 0 && qd.rows_per_seq <= qd.k_seq_rows))) {
+        if ((e = get_tensor_map(qd.vt_dst, (long long)seqs * qd.d, qd.vt_ld, qd.vt_ld, 64, 64, &mo.vt, 2)) != cudaSuccess) return e;
+        if (qd.k_dst != nullptr &&
+            (e = get_tensor_map(qd.k_dst, (long long)seqs * qd.k_seq_rows, qd.d, qd.d, BM, 64, &mo.k, 2)) != cudaSuccess) return e;
+        tma_out = 3;
+      }
     }
   }
   // CTA pairs on 256 x 256 tiles for the large GEMMs (bn_hint 512 forces them, SDD_GEMM_PAIR=0 switches them off, =2 drops the size rule)
@@ -1472,17 +1584,23 @@ cudaError_t launch_gemm_tc(const __nv_bfloat16* A, long long a_cap, const __nv_b
     const char* pe = getenv("SDD_GEMM_PAIR");
     const bool pair_on = pe == nullptr || atoi(pe) != 0;
     const bool pair_any_size = pe != nullptr && atoi(pe) == 2;      // tests: pairs wherever they are eligible
-    const bool eligible = !hilo && out_lo == nullptr && (M % 256) == 0 && (N % 256) == 0 && (bn_hint == 512 || bn == 256);
+    // ragged edges are clipped by the TMA stores' tensor maps; other epilogues take whole tiles only
+    const bool all_tma = tma_out == 1 || tma_out == 3 || tma_out == 5;
+    const bool eligible = (all_tma || (!hilo && out_lo == nullptr && (M % 256) == 0 && (N % 256) == 0)) && (bn_hint == 512 || bn == 256);
     if (bn_hint == 512 && !eligible) return cudaErrorInvalidValue;
-    // (forwards of a few thousand rows gain nothing from pairs; measured at 4608 rows: 3 to 5 % slower)
-    if (eligible && (bn_hint == 512 || (pair_on && splits == 1 && (M >= 8192 || pair_any_size) && mt * (N / 256) > 2 * SMS))) {
+    // Pairs win wherever there is more than one wave of their tiles (4096 x 4800 x 1600: 56.6 -> 45.9 us, 2304 x 3072 x 768:
+    // 19.4 -> 15.6); a single wave is better served by the one-tile kernel's deeper ring and K splits (512 x 4800 x 1600:
+    // 12.3 against 13.6 us).
+    const long long pair_tiles = (long long)((M + 255) / 256) * ((N + 255) / 256);
+    if (eligible && (bn_hint == 512 || (pair_on && splits == 1 && (pair_tiles > SMS / 2 || pair_any_size)))) {
       CUtensorMap mb_half;
       if ((e = get_tensor_map(W, N, K, K, 128, BK, &mb_half)) != cudaSuccess) return e;
-      const int tiles_m2 = M / 256, tiles_n = N / 256;
+      const int tiles_m2 = (M + 255) / 256, tiles_n = (N + 255) / 256;
       const long long tiles = (long long)tiles_m2 * tiles_n;
       const unsigned pairs = (unsigned)(tiles < SMS / 2 ? tiles : SMS / 2);
-      launch_k(gemm_tc_pair_kernel, dim3(2 * pairs), dim3(PAIR_THREADS), (size_t)PAIR_SMEM, st, ma, mb_half, mo, tma_out, M, N, K, epi,
-               bias, out, ldc, status, qd, skip, tiles_m2, tiles_n, (long long)N * K * 2 <= (48ll << 20) ? 1 : 0);
+      launch_k(hilo ? gemm_tc_pair_kernel<true> : gemm_tc_pair_kernel<false>, dim3(2 * pairs), dim3(PAIR_THREADS), (size_t)PAIR_SMEM, st, ma,
+               mb_half, ml, mo, tma_out, M, N, K, epi, bias, out, ldc, status, qd, skip, tiles_m2, tiles_n,
+               (long long)N * K * 2 <= (48ll << 20) ? 1 : 0);
       return cudaGetLastError();
     }
   }
