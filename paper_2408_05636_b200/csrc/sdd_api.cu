@@ -102,6 +102,7 @@ struct Buffers {
   float* h_s;                  // residual stream of the gamma slot rows [batch * gamma, d_q] (last drafter block)
   void* vt;                    // drafter V transposed [batch][d_q][lcap_max] (tensor-core path)
   void* kv;                    // target KV cache [layer][batch][n_ctx][2][d]
+  float* mlp_few;              // hidden layer of a forward of at most eight rows, fp32 [8][4 d]
 };
 
 struct Dims {
@@ -151,6 +152,7 @@ static size_t carve(const Dims& D, const Net& P, const Net& Q, uint8_t* base, Bu
   b.mlp_lo = take(mx(rq * Q.d, rp * P.d) * 4 * D.esize);
   b.xf_lo = take(Bn * (G + 1) * mx(Q.d, P.d) * D.esize);
   b.h_s = (float*)take(Bn * G * Q.d * 4);
+  b.mlp_few = (float*)take(8 * 4 * mx(Q.d, P.d) * 4);
   b.kv = take((size_t)P.n_layer * Bn * P.n_ctx * 2 * P.d * D.esize);
   if (B) *B = b;
   return off;
@@ -189,6 +191,7 @@ struct sdd_ctx {
   bool hilo;                   // SDD_HILO != 0 (default): hi/lo activation pairs in the target's MLP and LM head
   bool force_simt;             // SDD_GEMM=simt: run bf16 GEMMs on the CUDA-core kernel (cross-check)
   int bn_hint;                 // SDD_GEMM_BN: N tile of the tensor-core GEMM (0 = choose)
+  bool few_rows;               // SDD_FEW_ROWS != 0 (default): forwards of at most eight rows on the weight-streaming kernels
   bool head_stats;             // SDD_HEAD_STATS != 0 (default): soft-max statistics from the target LM head's epilogue
   bool use_graph;              // SDD_GRAPH != 0: sdd_step replays a captured graph per row-count bucket
   struct GraphEntry { cudaGraphExec_t exec; uint64_t launches; };
@@ -391,6 +394,30 @@ static int forward_drafter(sdd_ctx* c) {
   return SDD_OK;
 }
 
+// The blocks of a forward of at most eight rows (see sdd_decode.cu): five launches each, LayerNorm inside its consumer.
+static int run_blocks_few(sdd_ctx* c, const Net& N, void* kv, const int* len, int rows_per_seq, int gcat, int acat) {
+  const Buffers& B = c->B;
+  const int d = N.d, rows = c->D.batch * rows_per_seq;
+  const size_t layer_elems = (size_t)c->D.batch * N.n_ctx * 2 * d;
+  typedef __nv_bfloat16 bf;
+  for (int l = 0; l < N.n_layer; ++l) {
+    const Layer& L = N.layers[l];
+    bf* kc = (bf*)kv + (size_t)l * layer_elems;
+    QkvDst qd = {};
+    qd.k_dst = kc; qd.vt_dst = kc + layer_elems / 2; qd.ctx_len = len; qd.rows_per_seq = rows_per_seq; qd.mode = 1;
+    qd.d = d; qd.k_seq_rows = N.n_ctx; qd.vt_ld = N.n_ctx;
+    SDD_LAUNCH(c, gcat, launch_gemv_ln(B.h, L.ln1_g, L.ln1_b, (const bf*)L.w_qkv, L.b_qkv, rows, d, 3 * d, (bf*)B.qkv, nullptr, &qd,
+                                       &B.rs->status, c->st));
+    SDD_LAUNCH(c, acat, launch_attn_few((const bf*)B.qkv, 3 * d, kc, qd.vt_dst, (bf*)B.att, len, c->D.batch, rows_per_seq, N.n_ctx,
+                                        N.n_head, c->st));
+    SDD_LAUNCH(c, gcat, launch_gemv_add(B.att, false, (const bf*)L.w_o, L.b_o, rows, d, d, B.h, &B.rs->status, c->st));
+    SDD_LAUNCH(c, gcat, launch_gemv_ln(B.h, L.ln2_g, L.ln2_b, (const bf*)L.w_fc1, L.b_fc1, rows, d, 4 * d, nullptr, B.mlp_few, nullptr,
+                                       &B.rs->status, c->st));
+    SDD_LAUNCH(c, gcat, launch_gemv_add(B.mlp_few, true, (const bf*)L.w_fc2, L.b_fc2, rows, 4 * d, d, B.h, &B.rs->status, c->st));
+  }
+  return SDD_OK;
+}
+
 // Causal forward of network N over rows_per_seq new tokens per sequence against its KV cache `kv`; `len` holds the
 // per-sequence length that fixes the rows' positions (see TargetMode); the caller has written the embeddings to B.h.
 template <typename T>
@@ -405,6 +432,9 @@ static int forward_causal(sdd_ctx* c, const Net& N, void* kv, const int* len, in
   hilo = hilo && tc;
   // tensor-core path: per layer the cache is K [B][n_ctx][d] followed by V^T [B][d][n_ctx];
   // CUDA-core path: [B][n_ctx][K|V][d]
+  if (tc && mode == TARGET_VERIFY && c->few_rows && decode_fits(D.batch, rows_per_seq, N.d, N.d_head, N.n_ctx))
+    SDD_TRY(run_blocks_few(c, N, kv, len, rows_per_seq, gcat, acat));
+  else
   SDD_TRY((run_blocks<T>(c, N, rows, gcat, hilo, nullptr,
     [&](int l, QkvDst* qd) -> bool {
       if (!tc) return false;
@@ -627,6 +657,8 @@ int32_t sdd_create(const sdd_model* target, const sdd_model* drafter, const sdd_
     c->bn_hint = bn ? atoi(bn) : 0;
     const char* hs = getenv("SDD_HEAD_STATS");
     c->head_stats = hs == nullptr || atoi(hs) != 0;
+    const char* fr = getenv("SDD_FEW_ROWS");
+    c->few_rows = fr == nullptr || atoi(fr) != 0;
     const char* gr = getenv("SDD_GRAPH");
     // the legacy default stream cannot be captured: rounds are then enqueued kernel by kernel
     c->use_graph = (gr == nullptr || atoi(gr) != 0) && c->st != nullptr && c->st != cudaStreamLegacy;
@@ -648,6 +680,7 @@ int32_t sdd_create(const sdd_model* target, const sdd_model* drafter, const sdd_
   if (c->P.dtype == SDD_BF16) {   // before anything can be captured into a graph
     SDD_CUDA(tc_prepare_gemm());
     SDD_CUDA(tc_prepare_attn());
+    SDD_CUDA(prepare_decode());
   } else {
     SDD_CUDA(tc_prepare_gemm_f32());
   }

@@ -41,7 +41,7 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 // q: row 0 of the CTA's query rows (row stride q_ld), head's columns; k / v: key 0 (row stride kv_ld); rows past n_q are
 // not stored; query row i sees keys 0 .. min(n_keys, limit0 + i * limit_step) - 1
 template <typename T, int DH>
-__device__ __forceinline__ void attn_rows(const T* __restrict__ q, long long q_ld, const T* __restrict__ k, const T* __restrict__ v,
+__device__ __forceinline__ void attn_rows(const T* q, long long q_ld, const T* k, const T* v,
                                           long long kv_ld, int n_q, int n_keys, int limit0, int limit_step, T* __restrict__ out,
                                           int out_ld) {
   constexpr int ROW = fa_row<T, DH>(), QROW = fa_row<float, DH>(), PER16 = 16 / (int)sizeof(T), COLS = DH / 4;
@@ -182,8 +182,8 @@ __device__ __forceinline__ void attn_rows(const T* __restrict__ q, long long q_l
 
 template <typename T, int DH>
 __global__ void __launch_bounds__(FA_THREADS)
-attn_bidir_kernel(const T* __restrict__ qkv, T* __restrict__ out, const int* __restrict__ ctx_len, int gamma, int L_cap,
-                  int n_head, const int* __restrict__ skip) {
+attn_bidir_kernel(const T* qkv, T* __restrict__ out, const int* ctx_len, int gamma, int L_cap,
+                  int n_head, const int* skip) {
   pdl_launch_dependents();
   pdl_wait();
   if (skip != nullptr && *skip) return;
@@ -192,15 +192,15 @@ attn_bidir_kernel(const T* __restrict__ qkv, T* __restrict__ out, const int* __r
   const int L = ctx_len[b] + gamma;
   if (i0 >= L) return;                                       // padding rows are never read by valid ones; they stay as they are
   const long long row0 = (long long)b * L_cap;
-  const T* __restrict__ base = qkv + row0 * 3 * d + h * DH;
+  const T* base = qkv + row0 * 3 * d + h * DH;
   attn_rows<T, DH>(base + (long long)i0 * 3 * d, 3ll * d, base + d, base + 2 * d, 3ll * d, min(FA_Q, L - i0), L, L, 0,
                    out + (row0 + i0) * d + h * DH, d);
 }
 
 template <typename T, int DH>
 __global__ void __launch_bounds__(FA_THREADS)
-attn_cached_kernel(const T* __restrict__ qkv, const T* __restrict__ cache, T* __restrict__ out,
-                   const int* __restrict__ ctx_len, int rows_per_seq, int mode, int n_ctx, int n_head) {
+attn_cached_kernel(const T* qkv, const T* cache, T* __restrict__ out,
+                   const int* ctx_len, int rows_per_seq, int mode, int n_ctx, int n_head) {
   pdl_launch_dependents();
   pdl_wait();
   const int j0 = blockIdx.x * FA_Q, h = blockIdx.y, b = blockIdx.z;
@@ -212,7 +212,7 @@ attn_cached_kernel(const T* __restrict__ qkv, const T* __restrict__ cache, T* __
   int n_q = mode == TARGET_VERIFY ? min(rows_per_seq - j0, n_ctx - pos0) : min(rows_per_seq - j0, c - 1 - j0);
   n_q = min(n_q, FA_Q);
   if (n_q <= 0) return;
-  const T* __restrict__ kb = cache + (long long)b * n_ctx * 2 * d + h * DH;
+  const T* kb = cache + (long long)b * n_ctx * 2 * d + h * DH;
   attn_rows<T, DH>(qkv + row * 3 * d + h * DH, 3ll * d, kb, kb + d, 2ll * d, n_q, pos0 + n_q, pos0 + 1, 1, out + row * d + h * DH, d);
 }
 

@@ -154,6 +154,9 @@ __device__ __forceinline__ float gelu_tanh(float x) {
 // predecessor has triggered, hence is resident, so the resident CTAs are always a contiguous window of the chain
 // and nobody waits on a CTA that cannot be scheduled.  (2) Nothing ahead of the wait reads memory that a kernel of
 // the library writes (weights, LayerNorm gains: constant), except hints whose staleness costs time only.
+// The compiler must not break that rule either: a load through a const __restrict__ pointer counts as invariant and may be
+// moved above the wait, so kernels take such pointers only to memory that is constant (it did happen: a product that
+// normalised its input rows read them ahead of the kernel that was still adding to them).
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -101,7 +101,7 @@ template <int BN, bool SWAP>
 __global__ void __launch_bounds__(FX_THREADS)
 gemm_f32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int rows_a, int rows_b,
                 int K, int splits, int epi, const float* __restrict__ bias, float* __restrict__ out, int ldc, int* status,
-                const int* __restrict__ skip) {
+                const int* skip) {
   constexpr int FS = fx_f32_stages<BN>(), BS = fx_bf16_stages<BN>();
   constexpr int F_BYTES = fx_f32_bytes<BN>(), B_BYTES = fx_bf16_bytes<BN>();
   constexpr int BF_OFF = FS * F_BYTES, BAR_OFF = fx_bar_off<BN>();

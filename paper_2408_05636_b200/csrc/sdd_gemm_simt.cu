@@ -9,8 +9,8 @@ constexpr int SG_BM = 64, SG_BN = 64, SG_BK = 16, SG_THREADS = 256;
 using T = __nv_bfloat16;
 
 __global__ void __launch_bounds__(SG_THREADS)
-gemm_simt_kernel(const T* __restrict__ A, int lda, const T* __restrict__ W, const float* __restrict__ bias, int M, int N,
-                 int K, int epi, void* __restrict__ out, int ldc, const int* __restrict__ skip) {
+gemm_simt_kernel(const T* A, int lda, const T* __restrict__ W, const float* __restrict__ bias, int M, int N,
+                 int K, int epi, void* __restrict__ out, int ldc, const int* skip) {
   pdl_launch_dependents();
   pdl_wait();
   if (skip != nullptr && *skip) return;

@@ -673,7 +673,7 @@ __global__ void __launch_bounds__(one_tile_threads<BN, SWAP>())
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_lo, const __grid_constant__ OutMaps maps_out, int tma_out,
                int rows_a, int rows_b, int K, int epi, const float* __restrict__ bias, void* __restrict__ out,
-               void* __restrict__ out_lo, int ldc, int* status, const QkvDst qd, const int* __restrict__ skip) {
+               void* __restrict__ out_lo, int ldc, int* status, const QkvDst qd, const int* skip) {
 
   constexpr int STAGES = ring_stages<BN, SWAP, HILO, DEEP>();
   constexpr int STAGE_BYTES = stage_bytes<BN, SWAP, HILO>();
@@ -875,7 +875,7 @@ __global__ void __launch_bounds__(THREADS)
 gemm_tc_persist_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                        const __grid_constant__ CUtensorMap map_lo, const __grid_constant__ OutMaps maps_out, int tma_out,
                        int rows_a, int rows_b, int K, int epi, const float* __restrict__ bias, void* __restrict__ out,
-                       void* __restrict__ out_lo, int ldc, int* status, const QkvDst qd, const int* __restrict__ skip,
+                       void* __restrict__ out_lo, int ldc, int* status, const QkvDst qd, const int* skip,
                        int tiles_m, int tiles_n, int n_fastest, const HeadStats hs, int hs_chunks) {
   constexpr int STAGES = persist_stages<BN, HILO, SWAP>();
   constexpr int STAGE_BYTES = stage_bytes<BN, SWAP, HILO>();
@@ -1085,7 +1085,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PAIR_THREADS)
 gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                     const __grid_constant__ CUtensorMap map_lo, const __grid_constant__ OutMaps maps_out, int tma_out, int rows_a, int rows_b, int K, int epi,
                     const float* __restrict__ bias, void* __restrict__ out, int ldc, int* status, const QkvDst qd,
-                    const int* __restrict__ skip, int tiles_m2, int tiles_n, int n_fastest) {
+                    const int* skip, int tiles_m2, int tiles_n, int n_fastest) {
   constexpr int BN = 256;
   constexpr int STAGES = pair_stages<HILO>(), PAIR_STAGE_BYTES = pair_stage_bytes<HILO>();
   extern __shared__ uint8_t smem_raw[];

@@ -47,9 +47,9 @@ __device__ __forceinline__ void emb_layernorm_store(const float (&x)[EMB_MAX_PER
 
 template <typename T>
 __global__ void __launch_bounds__(EMB_THREADS)
-embed_drafter_kernel(const T* __restrict__ wte, const T* __restrict__ wpe, const int* __restrict__ tokens,
-                     int tok_stride, const int* __restrict__ ctx_len, const int* __restrict__ slot_ids,
-                     int gamma, int L_cap, int d, float* __restrict__ h, const int* __restrict__ skip,
+embed_drafter_kernel(const T* __restrict__ wte, const T* __restrict__ wpe, const int* tokens,
+                     int tok_stride, const int* ctx_len, const int* slot_ids,
+                     int gamma, int L_cap, int d, float* __restrict__ h, const int* skip,
                      const float* __restrict__ ln_g, const float* __restrict__ ln_b, T* __restrict__ xn, int vocab,
                      int* __restrict__ status) {
   pdl_launch_dependents();
@@ -92,8 +92,8 @@ embed_drafter_kernel(const T* __restrict__ wte, const T* __restrict__ wpe, const
 // target rows: sequence b owns rows b*rows_per_seq ..; VERIFY: row j = [last context token, drafts] at
 // position c-1+j; PREFILL: row j = context token j at position j (valid while j < c-1, else zero).
 template <typename T>
-__global__ void embed_target_kernel(const T* __restrict__ wte, const T* __restrict__ wpe, const int* __restrict__ tokens,
-                                    int tok_stride, const int* __restrict__ ctx_len, const int* __restrict__ slot_ids,
+__global__ void embed_target_kernel(const T* __restrict__ wte, const T* __restrict__ wpe, const int* tokens,
+                                    int tok_stride, const int* ctx_len, const int* slot_ids,
                                     int gamma, int rows_per_seq, int mode, int d, float* __restrict__ h, int vocab,
                                     int* __restrict__ status) {
   pdl_launch_dependents();
@@ -129,8 +129,8 @@ __global__ void embed_target_kernel(const T* __restrict__ wte, const T* __restri
 // evaluation's effective length c + off, which the other kernels of the evaluation take in place of ctx_len
 // (their rows then sit at positions eff - 1 + i, the convention of a verification forward).
 template <typename T>
-__global__ void embed_ar_kernel(const T* __restrict__ wte, const T* __restrict__ wpe, const int* __restrict__ tokens,
-                                int tok_stride, const int* __restrict__ ctx_len, const int* __restrict__ slot_ids,
+__global__ void embed_ar_kernel(const T* __restrict__ wte, const T* __restrict__ wpe, const int* tokens,
+                                int tok_stride, const int* ctx_len, const int* slot_ids,
                                 int gamma, int rows_per_seq, int off, int d, float* __restrict__ h,
                                 int* __restrict__ eff_len, int vocab, int* __restrict__ status) {
   pdl_launch_dependents();
@@ -162,7 +162,7 @@ constexpr int LN_MAX_PER_LANE = 64;  // d_model <= 2048
 constexpr float LN_EPS = 1e-5f;
 
 template <typename T>
-__device__ __forceinline__ void layernorm_row(const float* __restrict__ src, const float* __restrict__ g,
+__device__ __forceinline__ void layernorm_row(const float* src, const float* __restrict__ g,
                                               const float* __restrict__ bta, T* __restrict__ dst, T* __restrict__ dst_lo,
                                               int d) {
   const int lane = threadIdx.x & 31;
@@ -212,8 +212,8 @@ __device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16* p, float a,
 
 template <typename T, int NV>
 __global__ void __launch_bounds__(128)
-layernorm_vec_kernel(const float* __restrict__ h, const float* __restrict__ g, const float* __restrict__ bta,
-                     T* __restrict__ out, T* __restrict__ out_lo, long long rows, int d, const int* __restrict__ skip) {
+layernorm_vec_kernel(const float* h, const float* __restrict__ g, const float* __restrict__ bta,
+                     T* __restrict__ out, T* __restrict__ out_lo, long long rows, int d, const int* skip) {
   // gain and bias are weights (never written while the library runs): fetched before the wait for the kernel ahead
   const int lane = threadIdx.x & 31;
   float4 gg[NV], bb[NV];
@@ -227,7 +227,7 @@ layernorm_vec_kernel(const float* __restrict__ h, const float* __restrict__ g, c
   pdl_wait();
   const long long row = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
   if (row >= rows) return;
-  const float* __restrict__ src = h + row * d;
+  const float* src = h + row * d;
   // the row's loads are issued before the skip flag is looked at, so that the two round trips overlap
   float4 x[NV];
 #pragma unroll
@@ -267,8 +267,8 @@ layernorm_vec_kernel(const float* __restrict__ h, const float* __restrict__ g, c
 
 template <typename T>
 __global__ void __launch_bounds__(128)
-layernorm_kernel(const float* __restrict__ h, const float* __restrict__ g, const float* __restrict__ bta,
-                 T* __restrict__ out, T* __restrict__ out_lo, long long rows, int d, const int* __restrict__ skip) {
+layernorm_kernel(const float* h, const float* __restrict__ g, const float* __restrict__ bta,
+                 T* __restrict__ out, T* __restrict__ out_lo, long long rows, int d, const int* skip) {
   pdl_launch_dependents();
   pdl_wait();
   if (skip != nullptr && *skip) return;
@@ -279,9 +279,9 @@ layernorm_kernel(const float* __restrict__ h, const float* __restrict__ g, const
 
 template <typename T>
 __global__ void __launch_bounds__(128)
-layernorm_slots_kernel(const float* __restrict__ h, const float* __restrict__ g, const float* __restrict__ bta,
-                       T* __restrict__ out, const int* __restrict__ ctx_len, int batch, int gamma, int L_cap, int d,
-                       const int* __restrict__ skip) {
+layernorm_slots_kernel(const float* h, const float* __restrict__ g, const float* __restrict__ bta,
+                       T* __restrict__ out, const int* ctx_len, int batch, int gamma, int L_cap, int d,
+                       const int* skip) {
   pdl_launch_dependents();
   pdl_wait();
   if (skip != nullptr && *skip) return;
@@ -296,9 +296,9 @@ layernorm_slots_kernel(const float* __restrict__ h, const float* __restrict__ g,
 // the rest of that block runs on a compact copy: att_s[b*gamma + j] = att[b*L_cap + c_b + j], the same for h.
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void gather_slots_kernel(const T* __restrict__ att, const float* __restrict__ h, const int* __restrict__ ctx_len,
+__global__ void gather_slots_kernel(const T* att, const float* h, const int* ctx_len,
                                     int gamma, int L_cap, int d, T* __restrict__ att_s, float* __restrict__ h_s,
-                                    const int* __restrict__ skip) {
+                                    const int* skip) {
   pdl_launch_dependents();
   pdl_wait();
   if (skip != nullptr && *skip) return;
@@ -314,7 +314,7 @@ __global__ void gather_slots_kernel(const T* __restrict__ att, const float* __re
 // KV append: cache[b][pos][0] = K row, cache[b][pos][1] = V row
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void kv_append_kernel(const T* __restrict__ qkv, T* __restrict__ cache, const int* __restrict__ ctx_len,
+__global__ void kv_append_kernel(const T* qkv, T* __restrict__ cache, const int* ctx_len,
                                  int rows_per_seq, int mode, int n_ctx, int d) {
   pdl_launch_dependents();
   pdl_wait();
@@ -324,7 +324,7 @@ __global__ void kv_append_kernel(const T* __restrict__ qkv, T* __restrict__ cach
   if (mode == TARGET_VERIFY) pos = c - 1 + j;
   else { if (j >= c - 1) return; pos = j; }
   if (pos >= n_ctx) return;
-  const T* __restrict__ src = qkv + ((long long)b * rows_per_seq + j) * 3 * d + d;  // K then V, contiguous
+  const T* src = qkv + ((long long)b * rows_per_seq + j) * 3 * d + d;  // K then V, contiguous
   T* __restrict__ dst = cache + ((long long)b * n_ctx + pos) * 2 * d;
   for (int e = threadIdx.x; e < 2 * d; e += blockDim.x) dst[e] = src[e];
 }

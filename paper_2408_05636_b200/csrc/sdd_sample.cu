@@ -28,14 +28,14 @@ __host__ __device__ inline int stats_chunks(int V) { return (V + 3 + STATS_CHUNK
 
 template <bool GREEDY>
 __global__ void __launch_bounds__(STATS_THREADS)
-row_stats_kernel(const float* __restrict__ buf_a, long long rows_a, const float* __restrict__ buf_b, long long rows_b,
+row_stats_kernel(const float* buf_a, long long rows_a, const float* buf_b, long long rows_b,
                  int V, int chunks, float inv_tau_a, float inv_tau_b, float2* __restrict__ partial) {
   pdl_launch_dependents();
   pdl_wait();
   const long long row = blockIdx.x / chunks;
   const int chunk = blockIdx.x - (int)(row * chunks);
   const bool is_a = row < rows_a;
-  const float* __restrict__ buf = is_a ? buf_a : buf_b;
+  const float* buf = is_a ? buf_a : buf_b;
   const long long lrow = is_a ? row : row - rows_a;
   const float inv_tau = is_a ? inv_tau_a : inv_tau_b;
   const long long r0 = lrow * V, r1 = r0 + V;           // flat element range of this row
@@ -125,7 +125,7 @@ row_stats_kernel(const float* __restrict__ buf_a, long long rows_a, const float*
 // Merge of the per-chunk pairs of one row by a group of `tpr` consecutive lanes (a power of two up to 32; `sub` = the
 // lane's index in its group): the log-sum-exp of z, valid in every lane of the group.  All 32 lanes of the warp call it
 // together (the shuffles are warp-wide); a group whose row does not exist passes valid = false.
-__device__ __forceinline__ float merge_partials(const float2* __restrict__ p, int chunks, int tpr, int sub, bool valid) {
+__device__ __forceinline__ float merge_partials(const float2* p, int chunks, int tpr, int sub, bool valid) {
   float m = -INFINITY;
   if (valid)
     for (int c = sub; c < chunks; c += tpr) m = fmaxf(m, p[c].x);
@@ -139,7 +139,7 @@ __device__ __forceinline__ float merge_partials(const float2* __restrict__ p, in
   for (int o = tpr >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   return m + logf(s);
 }
-__device__ __forceinline__ int merge_partials_argmax(const float2* __restrict__ p, int chunks, int tpr, int sub, bool valid) {
+__device__ __forceinline__ int merge_partials_argmax(const float2* p, int chunks, int tpr, int sub, bool valid) {
   ArgMax a;
   a.s = -INFINITY;
   a.i = 0x7fffffff;
@@ -272,7 +272,7 @@ constexpr int SAMPLE_THREADS = 512;
 // src when greedy); the row z is stored to dst, log q(x) = z_x - logsumexp(z) to *logq_out and logsumexp(z) to
 // *lseq_out.  `mark` goes to
 // *reveal_out (the denoising step, or the evaluation index of an autoregressive drafter).
-__device__ __forceinline__ void draw_slot(const float* __restrict__ src, float* __restrict__ dst, int* __restrict__ slot_out,
+__device__ __forceinline__ void draw_slot(const float* src, float* __restrict__ dst, int* __restrict__ slot_out,
                                           float* __restrict__ logq_out, float* __restrict__ lseq_out,
                                           int* __restrict__ reveal_out, int j, int b, int V,
                                           int mark, float inv_tau_q, PhiloxKey key, uint32_t rnd, int* __restrict__ status) {
@@ -332,7 +332,7 @@ __device__ __forceinline__ void draw_slot(const float* __restrict__ src, float* 
   cl.sync();   // partials stay alive until rank 0 has read them
 }
 
-__device__ __forceinline__ bool unmask_sample_row(const float* __restrict__ step_logits,  // [B, gamma, V]
+__device__ __forceinline__ bool unmask_sample_row(const float* step_logits,  // [B, gamma, V]
                      int* __restrict__ slot_ids,             // [B, gamma]  (V = masked)
                      float* __restrict__ q_logits,           // [B, gamma, V]
                      float* __restrict__ logq,               // [B, gamma]
@@ -358,7 +358,7 @@ __device__ __forceinline__ bool unmask_sample_row(const float* __restrict__ step
 // evaluation would see the same input and reproduce the logits it already has, so its kernels are told to return
 // at once (the paper's "ddpm cache" strategy: a step without change costs no network evaluation).
 __global__ void __cluster_dims__(VC, 1, 1) __launch_bounds__(SAMPLE_THREADS)
-unmask_sample_kernel(const float* __restrict__ step_logits, int* __restrict__ slot_ids, float* __restrict__ q_logits,
+unmask_sample_kernel(const float* step_logits, int* __restrict__ slot_ids, float* __restrict__ q_logits,
                      float* __restrict__ logq, float* __restrict__ lseq, int* __restrict__ reveal_step, int gamma, int V, int k,
                      float inv_tau_q, PhiloxKey key, RoundState* __restrict__ rs, int cache_skip) {
   pdl_launch_dependents();
@@ -382,7 +382,7 @@ unmask_sample_kernel(const float* __restrict__ step_logits, int* __restrict__ sl
 // Draw of slot j by an autoregressive drafter (standard speculative decoding): the logits are the last of the
 // `rows_per_seq` rows the evaluation produced for each sequence; the slot is always written.  grid = (VC, batch).
 __global__ void __cluster_dims__(VC, 1, 1) __launch_bounds__(SAMPLE_THREADS)
-ar_sample_kernel(const float* __restrict__ logits, int rows_per_seq, int* __restrict__ slot_ids, float* __restrict__ q_logits,
+ar_sample_kernel(const float* logits, int rows_per_seq, int* __restrict__ slot_ids, float* __restrict__ q_logits,
                  float* __restrict__ logq, float* __restrict__ lseq, int* __restrict__ reveal_step, int gamma, int j, int V,
                  float inv_tau_q, PhiloxKey key, RoundState* __restrict__ rs) {
   pdl_launch_dependents();
@@ -406,9 +406,9 @@ constexpr int ACCEPT_THREADS = 256;
 
 // four CTAs per SM (64 registers): the stand-alone call's 8 x rows CTAs then fit in one wave for 64 rows
 __global__ void __cluster_dims__(VC, 1, 1) __launch_bounds__(ACCEPT_THREADS, 4)
-accept_kernel(const float* __restrict__ logits_p, const float* __restrict__ q_rows, const int* __restrict__ draft_ids,
-              const float* __restrict__ logq_in, const float* __restrict__ lseq_in, const float2* __restrict__ partial_p,
-              int chunks, const float2* __restrict__ partial_q, int chunks_q, int gamma, int V, float inv_tau_p,
+accept_kernel(const float* logits_p, const float* q_rows, const int* draft_ids,
+              const float* logq_in, const float* lseq_in, const float2* partial_p,
+              int chunks, const float2* partial_q, int chunks_q, int gamma, int V, float inv_tau_p,
               float inv_tau_q_rows, PhiloxKey key, uint32_t rnd_arg, RoundState* __restrict__ rs,
               float* __restrict__ accept_prob, int* __restrict__ n_accept, int* __restrict__ extra_token,
               int* __restrict__ out_ids) {
@@ -489,14 +489,14 @@ accept_kernel(const float* __restrict__ logits_p, const float* __restrict__ q_ro
   const int n = s_n;
 
   // extra token: residual of row n (n < gamma) or the bonus draw from row gamma
-  const float* __restrict__ prow = logits_p + ((long long)b * (gamma + 1) + n) * V;
+  const float* prow = logits_p + ((long long)b * (gamma + 1) + n) * V;
   const bool resid = n < gamma;
   ArgMax best, fallback;
   best.s = -INFINITY;
   best.i = 0x7fffffff;
   fallback = best;
   if (!greedy) {
-    const float* __restrict__ qrow = q_rows + ((long long)b * gamma + (resid ? n : 0)) * V;
+    const float* qrow = q_rows + ((long long)b * gamma + (resid ? n : 0)) * V;
     const float lsep = s_lsep[n];
     float lseq = 0.f;
     if (resid) {
@@ -588,8 +588,8 @@ accept_kernel(const float* __restrict__ logits_p, const float* __restrict__ q_ro
 // one block; host_mirror (mapped pinned memory, may be null) = [stamp, ctx_len[B], n_emitted[B], stamp]
 // ---------------------------------------------------------------------------------------------
 __global__ void commit_kernel(int* __restrict__ tokens, int tok_stride, int* __restrict__ ctx_len,
-                              int* __restrict__ n_emitted, const int* __restrict__ slot_ids,
-                              const int* __restrict__ n_accept, const int* __restrict__ extra_token, int batch, int gamma,
+                              int* __restrict__ n_emitted, const int* slot_ids,
+                              const int* n_accept, const int* extra_token, int batch, int gamma,
                               int max_new, RoundState* rs, int* __restrict__ out_ids, int* __restrict__ n_out,
                               volatile int* host_mirror) {
   pdl_launch_dependents();
