@@ -102,7 +102,6 @@ struct Buffers {
   float* h_s;                  // residual stream of the gamma slot rows [batch * gamma, d_q] (last drafter block)
   void* vt;                    // drafter V transposed [batch][d_q][lcap_max] (tensor-core path)
   void* kv;                    // target KV cache [layer][batch][n_ctx][2][d]
-  float* mlp_few;              // hidden layer of a forward of at most eight rows, fp32 [8][4 d]
 };
 
 struct Dims {
@@ -152,7 +151,6 @@ static size_t carve(const Dims& D, const Net& P, const Net& Q, uint8_t* base, Bu
   b.mlp_lo = take(mx(rq * Q.d, rp * P.d) * 4 * D.esize);
   b.xf_lo = take(Bn * (G + 1) * mx(Q.d, P.d) * D.esize);
   b.h_s = (float*)take(Bn * G * Q.d * 4);
-  b.mlp_few = (float*)take(8 * 4 * mx(Q.d, P.d) * 4);
   b.kv = take((size_t)P.n_layer * Bn * P.n_ctx * 2 * P.d * D.esize);
   if (B) *B = b;
   return off;
@@ -177,6 +175,7 @@ struct sdd_ctx {
   int* mirror_dev;
   std::vector<cudaEvent_t> ev;
   int runahead;
+  int key_splits;              // CTAs a head's keys are spread over in few-row attention (1, 2 or 4)
   int lcap;                    // padded rows per sequence of the current round's drafter forwards
   size_t act_elems, xf_elems;  // capacity (elements) of the xn / att buffers (mlp: 4x) and of xf
   Net A;                       // autoregressive drafter of the speculative-decoding warm start (sdd_sps_attach)
@@ -191,7 +190,7 @@ struct sdd_ctx {
   bool hilo;                   // SDD_HILO != 0 (default): hi/lo activation pairs in the target's MLP and LM head
   bool force_simt;             // SDD_GEMM=simt: run bf16 GEMMs on the CUDA-core kernel (cross-check)
   int bn_hint;                 // SDD_GEMM_BN: N tile of the tensor-core GEMM (0 = choose)
-  bool few_rows;               // SDD_FEW_ROWS != 0 (default): forwards of at most eight rows on the weight-streaming kernels
+  int few_rows;                // SDD_FEW_ROWS (default 32): causal forwards of at most this many rows run on the weight-streaming kernels
   bool head_stats;             // SDD_HEAD_STATS != 0 (default): soft-max statistics from the target LM head's epilogue
   bool use_graph;              // SDD_GRAPH != 0: sdd_step replays a captured graph per row-count bucket
   struct GraphEntry { cudaGraphExec_t exec; uint64_t launches; };
@@ -394,26 +393,41 @@ static int forward_drafter(sdd_ctx* c) {
   return SDD_OK;
 }
 
-// The blocks of a forward of at most eight rows (see sdd_decode.cu): five launches each, LayerNorm inside its consumer.
-static int run_blocks_few(sdd_ctx* c, const Net& N, void* kv, const int* len, int rows_per_seq, int gcat, int acat) {
+// The blocks of a forward of a few rows (see sdd_decode.cu): LayerNorm inside its consumer for one or two rows
+static int run_blocks_few(sdd_ctx* c, const Net& N, void* kv, const int* len, int rows_per_seq, bool hilo, int gcat, int acat) {
   const Buffers& B = c->B;
   const int d = N.d, rows = c->D.batch * rows_per_seq;
   const size_t layer_elems = (size_t)c->D.batch * N.n_ctx * 2 * d;
   typedef __nv_bfloat16 bf;
+  int* status = &B.rs->status;
+  bf *qkv = (bf*)B.qkv, *att = (bf*)B.att, *xn = (bf*)B.xn, *xn_lo = (bf*)B.xn_lo, *mlp = (bf*)B.mlp, *mlp_lo = (bf*)B.mlp_lo;
   for (int l = 0; l < N.n_layer; ++l) {
     const Layer& L = N.layers[l];
     bf* kc = (bf*)kv + (size_t)l * layer_elems;
     QkvDst qd = {};
     qd.k_dst = kc; qd.vt_dst = kc + layer_elems / 2; qd.ctx_len = len; qd.rows_per_seq = rows_per_seq; qd.mode = 1;
     qd.d = d; qd.k_seq_rows = N.n_ctx; qd.vt_ld = N.n_ctx;
-    SDD_LAUNCH(c, gcat, launch_gemv_ln(B.h, L.ln1_g, L.ln1_b, (const bf*)L.w_qkv, L.b_qkv, rows, d, 3 * d, (bf*)B.qkv, nullptr, &qd,
-                                       &B.rs->status, c->st));
-    SDD_LAUNCH(c, acat, launch_attn_few((const bf*)B.qkv, 3 * d, kc, qd.vt_dst, (bf*)B.att, len, c->D.batch, rows_per_seq, N.n_ctx,
-                                        N.n_head, c->st));
-    SDD_LAUNCH(c, gcat, launch_gemv_add(B.att, false, (const bf*)L.w_o, L.b_o, rows, d, d, B.h, &B.rs->status, c->st));
-    SDD_LAUNCH(c, gcat, launch_gemv_ln(B.h, L.ln2_g, L.ln2_b, (const bf*)L.w_fc1, L.b_fc1, rows, d, 4 * d, nullptr, B.mlp_few, nullptr,
-                                       &B.rs->status, c->st));
-    SDD_LAUNCH(c, gcat, launch_gemv_add(B.mlp_few, true, (const bf*)L.w_fc2, L.b_fc2, rows, 4 * d, d, B.h, &B.rs->status, c->st));
+    if (rows <= 2) {
+      SDD_LAUNCH(c, gcat, launch_gemv_ln(B.h, L.ln1_g, L.ln1_b, (const bf*)L.w_qkv, L.b_qkv, rows, d, 3 * d, qkv, nullptr, &qd, status, c->st));
+    } else {
+      SDD_LAUNCH(c, CAT_LAYERNORM, launch_layernorm<bf>(B.h, L.ln1_g, L.ln1_b, xn, rows, d, c->st));
+      SDD_LAUNCH(c, gcat, launch_stream_gemm(xn, nullptr, (const bf*)L.w_qkv, L.b_qkv, rows, d, 3 * d, EPI_QKV, qkv, nullptr, &qd, status, c->st));
+    }
+    if (attn_few_fits(rows_per_seq, N.n_ctx))
+      SDD_LAUNCH(c, acat, launch_attn_few(qkv, 3 * d, kc, qd.vt_dst, att, len, c->D.batch, rows_per_seq, N.n_ctx, N.n_head, c->key_splits, c->st));
+    else
+      SDD_LAUNCH(c, acat, launch_attn_tc(qkv, (long long)(c->act_elems / d), 3 * d, 0, kc, (long long)c->D.batch * N.n_ctx, d, 0, N.n_ctx,
+                                         qd.vt_dst, N.n_ctx, att, d, len, c->D.batch, N.n_head, d, c->D.gamma, 1, rows_per_seq, status, c->st));
+    SDD_LAUNCH(c, gcat, launch_stream_gemm(att, nullptr, (const bf*)L.w_o, L.b_o, rows, d, d, EPI_RESIDUAL, B.h, nullptr, nullptr, status, c->st));
+    if (rows <= 2) {
+      SDD_LAUNCH(c, gcat, launch_gemv_ln(B.h, L.ln2_g, L.ln2_b, (const bf*)L.w_fc1, L.b_fc1, rows, d, 4 * d, mlp, mlp_lo, nullptr, status, c->st));
+    } else {
+      SDD_LAUNCH(c, CAT_LAYERNORM, launch_layernorm<bf>(B.h, L.ln2_g, L.ln2_b, xn, rows, d, c->st, hilo ? xn_lo : nullptr));
+      SDD_LAUNCH(c, gcat, launch_stream_gemm(xn, hilo ? xn_lo : nullptr, (const bf*)L.w_fc1, L.b_fc1, rows, d, 4 * d, EPI_GELU, mlp, mlp_lo, nullptr,
+                                             status, c->st));
+    }
+    SDD_LAUNCH(c, gcat, launch_stream_gemm(mlp, hilo || rows <= 2 ? mlp_lo : nullptr, (const bf*)L.w_fc2, L.b_fc2, rows, 4 * d, d, EPI_RESIDUAL, B.h,
+                                           nullptr, nullptr, status, c->st));
   }
   return SDD_OK;
 }
@@ -432,8 +446,8 @@ static int forward_causal(sdd_ctx* c, const Net& N, void* kv, const int* len, in
   hilo = hilo && tc;
   // tensor-core path: per layer the cache is K [B][n_ctx][d] followed by V^T [B][d][n_ctx];
   // CUDA-core path: [B][n_ctx][K|V][d]
-  if (tc && mode == TARGET_VERIFY && c->few_rows && decode_fits(D.batch, rows_per_seq, N.d, N.d_head, N.n_ctx))
-    SDD_TRY(run_blocks_few(c, N, kv, len, rows_per_seq, gcat, acat));
+  if (tc && mode == TARGET_VERIFY && rows <= c->few_rows && few_rows_fit((int)rows, N.d, N.d_head))
+    SDD_TRY(run_blocks_few(c, N, kv, len, rows_per_seq, hilo, gcat, acat));
   else
   SDD_TRY((run_blocks<T>(c, N, rows, gcat, hilo, nullptr,
     [&](int l, QkvDst* qd) -> bool {
@@ -516,9 +530,9 @@ static int forward_ar_drafter(sdd_ctx* c, int gamma, int j) {
   return SDD_OK;
 }
 
-// refresh the host's upper bound of every context length from the pinned mirror and pick the
-// padded row count of this round's drafter forwards
-static void choose_lcap(sdd_ctx* c) {
+// refresh the host's upper bound of every context length from the pinned mirror; what follows from the largest of them: the
+// padded row count of this round's drafter forwards, and over how many CTAs a head's keys are spread in few-row attention
+static void refresh_bounds(sdd_ctx* c) {
   const int Bn = c->D.batch;
   // the commit kernel writes head stamp, body, tail stamp; a reader therefore takes the tail first and the head
   // last: equal stamps then bracket a body that no writer touched in between
@@ -546,6 +560,10 @@ static void choose_lcap(sdd_ctx* c) {
   int lcap = (int)align_up((size_t)(cmax + c->D.gamma), ROW_TILE);
   if (lcap > c->D.lcap_max) lcap = c->D.lcap_max;
   c->lcap = lcap;
+  // (one row of the XL target at 512 keys: 1.29 ms a token on one CTA a head, 1.19 on four; at 100 keys the cluster costs more
+  // than it gives, 4.11 against 3.64 ms a warm-start round)
+  const int keys = cmax + c->D.gamma;
+  c->key_splits = keys <= 192 ? 1 : keys <= 384 ? 2 : 4;
 }
 
 template <typename T>
@@ -638,6 +656,7 @@ int32_t sdd_create(const sdd_model* target, const sdd_model* drafter, const sdd_
   c->ar_kv = nullptr;
   c->ar_eff = nullptr;
   c->sps_allowed = true;
+  c->key_splits = 1;
   c->profiling = false;
   c->prof_used = 0;
   {
@@ -658,7 +677,7 @@ int32_t sdd_create(const sdd_model* target, const sdd_model* drafter, const sdd_
     const char* hs = getenv("SDD_HEAD_STATS");
     c->head_stats = hs == nullptr || atoi(hs) != 0;
     const char* fr = getenv("SDD_FEW_ROWS");
-    c->few_rows = fr == nullptr || atoi(fr) != 0;
+    c->few_rows = fr == nullptr ? 32 : atoi(fr);
     const char* gr = getenv("SDD_GRAPH");
     // the legacy default stream cannot be captured: rounds are then enqueued kernel by kernel
     c->use_graph = (gr == nullptr || atoi(gr) != 0) && c->st != nullptr && c->st != cudaStreamLegacy;
@@ -749,7 +768,7 @@ static int round_prologue(sdd_ctx* c) {
   // bound the host's run-ahead so that the length mirror stays fresh
   if (c->rounds >= (uint64_t)c->runahead)
     SDD_CUDA(cudaEventSynchronize(c->ev[(c->rounds - c->runahead) % c->ev.size()]));
-  choose_lcap(c);
+  refresh_bounds(c);
   return SDD_OK;
 }
 static int enqueue_draft_begin(sdd_ctx* c) {
@@ -814,7 +833,8 @@ int32_t sdd_step(sdd_ctx* c, int32_t* out_ids, int32_t* n_out) {
   SDD_TRY(round_prologue(c));
   // per-launch timing: the event pairs are captured into a one-off graph, so the stamps are taken on the device
   // timeline without host launch gaps in between
-  const auto key = std::make_tuple(c->profiling ? -c->lcap - (int)c->prof_graphs.size() - 1 : c->lcap, (void*)out_ids,
+  const int few = attn_few_fits(c->D.gamma + 1, c->P.n_ctx) ? c->key_splits : 0;
+  const auto key = std::make_tuple(c->profiling ? -c->lcap - (int)c->prof_graphs.size() - 1 : c->lcap + few, (void*)out_ids,
                                    (void*)n_out);
   auto it = c->graphs.find(key);
   if (it == c->graphs.end()) {
@@ -848,13 +868,12 @@ int32_t sdd_ar_step(sdd_ctx* c, int32_t* out_ids, int32_t* n_out) {
   if (c == nullptr) return SDD_E_ARG;
   if (c->steps_done != -1) return SDD_E_STATE;
   c->sps_allowed = false;
-  if (c->rounds >= (uint64_t)c->runahead)
-    SDD_CUDA(cudaEventSynchronize(c->ev[(c->rounds - c->runahead) % c->ev.size()]));
+  SDD_TRY(round_prologue(c));
   if (!c->use_graph || c->profiling) {
     SDD_TRY(enqueue_verify_accept(c, 0, out_ids, n_out));
     return round_epilogue(c, 1);
   }
-  const auto key = std::make_tuple(0, (void*)out_ids, (void*)n_out);   // row count 0 never names a SpecDiff round
+  const auto key = std::make_tuple(c->key_splits, (void*)out_ids, (void*)n_out);   // below every padded row count
   auto it = c->graphs.find(key);
   if (it == c->graphs.end()) {
     const uint64_t l0 = c->launches;
@@ -948,14 +967,13 @@ int32_t sdd_sps_step(sdd_ctx* c, int32_t gamma_sps, int32_t* out_ids, int32_t* n
   if (c == nullptr) return SDD_E_ARG;
   if (!c->has_ar || !c->sps_allowed || c->steps_done != -1) return SDD_E_STATE;
   if (gamma_sps < 1 || gamma_sps > c->D.gamma) return SDD_E_ARG;
-  if (c->rounds >= (uint64_t)c->runahead)
-    SDD_CUDA(cudaEventSynchronize(c->ev[(c->rounds - c->runahead) % c->ev.size()]));
+  SDD_TRY(round_prologue(c));
   if (!c->use_graph || c->profiling) {
     SDD_TRY(enqueue_sps_round(c, gamma_sps, out_ids, n_out));
     return round_epilogue(c, gamma_sps + 1);
   }
-  // keys of the other graphs: padded row counts (positive), 0 (autoregressive step), small negative (timing passes)
-  const auto key = std::make_tuple(-(1 << 24) - gamma_sps, (void*)out_ids, (void*)n_out);
+  // keys of the other graphs: padded row counts, 1 to 4 (autoregressive step), small negative (timing passes)
+  const auto key = std::make_tuple(-(1 << 24) - gamma_sps * 8 - c->key_splits, (void*)out_ids, (void*)n_out);
   auto it = c->graphs.find(key);
   if (it == c->graphs.end()) {
     const uint64_t l0 = c->launches;
@@ -984,7 +1002,7 @@ int32_t sdd_progress(sdd_ctx* c, uint64_t* rounds_done, int32_t* min_emitted) {
   const int Bn = c->D.batch;
   volatile int* m = c->mirror;
   for (int attempt = 0; attempt < 64; ++attempt) {
-    // tail stamp, body, head stamp: the reverse of the commit kernel's write order (see choose_lcap)
+    // tail stamp, body, head stamp: the reverse of the commit kernel's write order (see refresh_bounds)
     const int s1 = m[1 + 2 * Bn];
     std::atomic_thread_fence(std::memory_order_acquire);
     int mn = 0x7fffffff;

@@ -155,19 +155,22 @@ cudaError_t launch_attn_tc(const __nv_bfloat16* q, long long q_rows_total, int q
                            int gamma, int mode, int q_rows_per_seq, int* status, cudaStream_t st,
                            const int* skip = nullptr);
 
-// ---- forwards of at most eight token rows, bf16 (sdd_decode.cu) --------------------------------
-bool decode_fits(int batch, int rows_per_seq, int d, int d_head, int n_ctx);
+// ---- forwards of a few token rows, bf16, d_head 64 (sdd_decode.cu) -----------------------------
+bool few_rows_fit(int M, int d, int d_head);
+bool attn_few_fits(int R, int n_ctx);
 cudaError_t prepare_decode();
-// out = epilogue(LayerNorm(h) W^T + bias): qkv given: Q to out_q (row stride N), K and V^T to the caches (verify positions);
-// else GELU to out_f (fp32, row stride N)
+// M = 1 or 2: out = epilogue(LayerNorm(h) W^T + bias); qkv given: Q to out (row stride N), K and V^T to the caches (verify
+// positions); else GELU as a hi/lo pair to out / out_lo (row stride N)
 cudaError_t launch_gemv_ln(const float* h, const float* ln_g, const float* ln_b, const __nv_bfloat16* W, const float* bias, int M, int K,
-                           int N, __nv_bfloat16* out_q, float* out_f, const QkvDst* qkv, int* status, cudaStream_t st);
-// h += x W^T + bias, x bf16 or fp32 with row stride K
-cudaError_t launch_gemv_add(const void* x, bool x_f32, const __nv_bfloat16* W, const float* bias, int M, int K, int N, float* h,
-                            int* status, cudaStream_t st);
-// attention of R <= 8 rows per sequence at positions ctx_len[b] - 1 + r; kc [batch][n_ctx][d], vt [batch][d][n_ctx]
+                           int N, __nv_bfloat16* out, __nv_bfloat16* out_lo, const QkvDst* qkv, int* status, cudaStream_t st);
+// M <= 32: epilogue((x + x_lo) W^T + bias), x row stride K, x_lo may be null; EPI_RESIDUAL adds to out (fp32, row stride N),
+// EPI_GELU and EPI_QKV as above
+cudaError_t launch_stream_gemm(const __nv_bfloat16* x, const __nv_bfloat16* x_lo, const __nv_bfloat16* W, const float* bias, int M, int K, int N,
+                               int epi, void* out, __nv_bfloat16* out_lo, const QkvDst* qkv, int* status, cudaStream_t st);
+// attention of R <= 8 rows per sequence at positions ctx_len[b] - 1 + r; kc [batch][n_ctx][d], vt [batch][d][n_ctx];
+// key_splits: 1, 2 or 4 CTAs share a head's keys
 cudaError_t launch_attn_few(const __nv_bfloat16* q, int q_ld, const __nv_bfloat16* kc, const __nv_bfloat16* vt, __nv_bfloat16* out,
-                            const int* ctx_len, int batch, int R, int n_ctx, int n_head, cudaStream_t st);
+                            const int* ctx_len, int batch, int R, int n_ctx, int n_head, int key_splits, cudaStream_t st);
 
 // ---- attention (sdd_attn.cu) ----------------------------------------------------------------
 cudaError_t prepare_attn();   // one-time set-up, as above
