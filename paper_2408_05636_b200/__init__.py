@@ -107,6 +107,20 @@ def lib() -> C.CDLL:
     return _lib
 
 
+_native = None
+
+
+def native():
+    """The native call path for torch tensors (built next to libsdd.so); raises if it has not been built."""
+    global _native
+    if _native is None:
+        import importlib
+        _torch()
+        lib()
+        _native = importlib.import_module("._sdd_torch", __name__)
+    return _native
+
+
 def _check(status: int, where: str):
     if status != SDD_OK:
         raise SddError(status, where)
@@ -158,23 +172,10 @@ def sdd_accept_logits(logits_p, logits_q, draft_ids, temp_p: float, temp_q: floa
                       scratch=None, stream=None):
     """logits_p [rows, gamma+1, V] fp32, logits_q [rows, gamma, V] fp32, draft_ids [rows, gamma] int32, all CUDA
     tensors.  Returns (n_accept [rows], out_ids [rows, gamma+1], accept_prob [rows, gamma])."""
-    torch = _torch()
-    rows, g1, V = logits_p.shape
-    gamma = g1 - 1
-    assert logits_q.shape == (rows, gamma, V) and draft_ids.shape == (rows, gamma)
-    assert logits_p.is_contiguous() and logits_q.is_contiguous() and draft_ids.is_contiguous()
-    assert logits_p.dtype == torch.float32 and logits_q.dtype == torch.float32 and draft_ids.dtype == torch.int32
-    dev = logits_p.device
-    n_accept = torch.empty(rows, dtype=torch.int32, device=dev)
-    out_ids = torch.empty(rows, gamma + 1, dtype=torch.int32, device=dev)
-    prob = torch.empty(rows, gamma, dtype=torch.float32, device=dev)
-    if scratch is None:
-        scratch = torch.empty(sdd_accept_scratch_bytes(rows, gamma, V), dtype=torch.uint8, device=dev)
-    st = stream if stream is not None else torch.cuda.current_stream(dev)
-    _check(lib().sdd_accept_logits(logits_p.data_ptr(), logits_q.data_ptr(), draft_ids.data_ptr(), rows, gamma, V,
-                                   float(temp_p), float(temp_q), int(seed), int(rnd), n_accept.data_ptr(),
-                                   out_ids.data_ptr(), prob.data_ptr(), scratch.data_ptr(), st.cuda_stream),
-           "sdd_accept_logits")
+    status, n_accept, out_ids, prob = (_native or native()).accept_logits(
+        logits_p, logits_q, draft_ids, temp_p, temp_q, seed, rnd, scratch, None if stream is None else stream.cuda_stream)
+    if status != SDD_OK:
+        raise SddError(status, "sdd_accept_logits")
     return n_accept, out_ids, prob
 
 
@@ -188,20 +189,10 @@ def sdd_accept_logits_static(logits_p, logits_q, draft_ids, n_accept, out_ids, a
     (n_accept [rows] int32, out_ids [rows, gamma+1] int32, accept_prob [rows, gamma] fp32).  Problems whose
     statistics do not fit ACCEPT_STATIC_SCRATCH_BYTES raise SddError(SDD_E_WORKSPACE).  Calls that may overlap on
     the GPU share the scratch and race; make the first call on a device outside stream capture."""
-    torch = _torch()
-    rows, g1, V = logits_p.shape
-    gamma = g1 - 1
-    assert logits_q.shape == (rows, gamma, V) and draft_ids.shape == (rows, gamma)
-    assert n_accept.shape == (rows,) and out_ids.shape == (rows, gamma + 1) and accept_prob.shape == (rows, gamma)
-    for t in (logits_p, logits_q, draft_ids, n_accept, out_ids, accept_prob):
-        assert t.is_cuda and t.is_contiguous()
-    assert logits_p.dtype == torch.float32 and logits_q.dtype == torch.float32 and accept_prob.dtype == torch.float32
-    assert draft_ids.dtype == torch.int32 and n_accept.dtype == torch.int32 and out_ids.dtype == torch.int32
-    st = stream if stream is not None else torch.cuda.current_stream(logits_p.device)
-    _check(lib().sdd_accept_logits_static(logits_p.data_ptr(), logits_q.data_ptr(), draft_ids.data_ptr(), rows, gamma,
-                                          V, float(temp_p), float(temp_q), int(seed), int(rnd), n_accept.data_ptr(),
-                                          out_ids.data_ptr(), accept_prob.data_ptr(), st.cuda_stream),
-           "sdd_accept_logits_static")
+    status = (_native or native()).accept_logits_static(logits_p, logits_q, draft_ids, n_accept, out_ids, accept_prob, temp_p, temp_q,
+                                                        seed, rnd, None if stream is None else stream.cuda_stream)
+    if status != SDD_OK:
+        raise SddError(status, "sdd_accept_logits_static")
 
 
 def sdd_debug_gemm_bf16(A, W, bias, M: int, epilogue: int, out, n_tile: int = 0, use_tensor_cores: bool = True,

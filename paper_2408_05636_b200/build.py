@@ -1,16 +1,20 @@
-"""Builds the CUDA library in-tree: csrc/*.cu -> libsdd.so (sm_100a only)."""
+"""Builds in-tree: csrc/*.cu -> libsdd.so (sm_100a only), csrc_torch/sdd_torch.cpp -> _sdd_torch (the native call path of the
+stand-alone acceptance step for torch tensors, linked against libsdd.so)."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libsdd.so")
 OBJ_DIR = os.path.join(HERE, "_build")
+TORCH_SRC = os.path.join(HERE, "csrc_torch", "sdd_torch.cpp")
+TORCH_OUT = os.path.join(HERE, "_sdd_torch" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
@@ -33,7 +37,26 @@ def _deps_mtime() -> float:
 
 
 def up_to_date() -> bool:
-    return os.path.exists(OUT) and os.path.getmtime(OUT) >= _deps_mtime()
+    return os.path.exists(OUT) and os.path.getmtime(OUT) >= _deps_mtime() and _torch_up_to_date()
+
+
+def _torch_up_to_date() -> bool:
+    deps = [TORCH_SRC, os.path.join(HERE, "..", "include", "sdd.h")]
+    return os.path.exists(TORCH_OUT) and os.path.getmtime(TORCH_OUT) >= max(os.path.getmtime(p) for p in deps)
+
+
+def _build_torch() -> None:
+    import torch
+    from torch.utils import cpp_extension as ext
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", TORCH_SRC, "-o", TORCH_OUT,
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f"-I{sysconfig.get_paths()['include']}"]
+    cmd += [f"-I{p}" for p in ext.include_paths()] + ["-I/usr/local/cuda/include"]
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cmd += [f"-L{lib}", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda", f"-L{HERE}", "-l:libsdd.so", "-L/usr/local/cuda/lib64", "-lcudart",
+            "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed on {TORCH_SRC}:\n{r.stdout}\n{r.stderr}")
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -59,6 +82,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
     r = subprocess.run([nvcc, "-shared", "-o", OUT, *objs, "-lcudart"], capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
+    if force or not _torch_up_to_date():
+        _build_torch()
     return OUT
 
 

@@ -52,14 +52,10 @@ extern "C" int32_t sdd_accept_logits_static(const float* logits_p, const float* 
   if (s != SDD_OK) return s;
   cudaStream_t st = (cudaStream_t)stream;
   const float itp = temp_p > 0.f ? 1.f / temp_p : 0.f, itq = temp_q > 0.f ? 1.f / temp_q : 0.f;
-  float2* partial = (float2*)scratch;
-  const long long rows_p = (long long)rows * (gamma + 1), rows_q = (long long)rows * gamma;
-  // every (row, chunk) pair that the second kernel reads is written by the first one in this same call,
-  // so nothing in the shared array has to be cleared between calls
-  if (launch_row_stats(logits_p, rows_p, logits_q, itp == 0.f ? 0 : rows_q, V, itp, itq, partial, st) != cudaSuccess)
-    return SDD_E_CUDA;
-  if (launch_accept(logits_p, logits_q, draft_ids, nullptr, nullptr, partial, chunks, partial + rows_p * chunks, chunks, rows, gamma, V, itp, itq,
-                    make_key(seed), (uint32_t)round, nullptr, accept_prob, n_accept, nullptr, out_ids, st) != cudaSuccess)
+  // every (row, chunk) pair that is read is written earlier in this same call, so nothing in the shared array has to be
+  // cleared between calls
+  if (launch_accept_standalone(logits_p, logits_q, draft_ids, rows, gamma, V, itp, itq, make_key(seed), (uint32_t)round, n_accept, out_ids,
+                               accept_prob, (float2*)scratch, st) != cudaSuccess)
     return SDD_E_CUDA;
   return SDD_OK;
 }

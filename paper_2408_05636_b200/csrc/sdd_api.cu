@@ -560,10 +560,10 @@ static void refresh_bounds(sdd_ctx* c) {
   int lcap = (int)align_up((size_t)(cmax + c->D.gamma), ROW_TILE);
   if (lcap > c->D.lcap_max) lcap = c->D.lcap_max;
   c->lcap = lcap;
-  // (one row of the XL target at 512 keys: 1.29 ms a token on one CTA a head, 1.19 on four; at 100 keys the cluster costs more
+  // (one row of the XL target at 512 keys: 1.27 ms a token on one CTA a head, 1.20 on two; at 100 keys the cluster costs more
   // than it gives, 4.11 against 3.64 ms a warm-start round)
   const int keys = cmax + c->D.gamma;
-  c->key_splits = keys <= 192 ? 1 : keys <= 384 ? 2 : 4;
+  c->key_splits = keys <= 192 ? 1 : keys <= 768 ? 2 : 4;
 }
 
 template <typename T>
@@ -594,9 +594,8 @@ static int verify_accept_t(sdd_ctx* c, int gamma, int32_t* out_ids, int32_t* n_o
                                    B.partial_p, c->st));
     chunks = D.chunks;
   }
-  SDD_LAUNCH(c, CAT_ACCEPT, launch_accept(B.logits_p, B.q_logits, B.slot_ids, B.logq, B.lse_q, B.partial_p, chunks, nullptr, 0, D.batch, gamma, D.V,
-                              c->inv_tau_p, c->inv_tau_p == 0.f ? 0.f : 1.f, c->key, 0u, B.rs, B.accept_prob, B.n_accept,
-                              B.extra_token, nullptr, c->st));
+  SDD_LAUNCH(c, CAT_ACCEPT, launch_accept(B.logits_p, B.q_logits, B.slot_ids, B.logq, B.lse_q, B.partial_p, chunks, D.batch, gamma, D.V,
+                              c->inv_tau_p, c->key, B.rs, B.accept_prob, B.n_accept, B.extra_token, c->st));
   SDD_LAUNCH(c, CAT_COMMIT, launch_commit(B.tokens, D.tok_stride, B.ctx_len, B.n_emitted, B.slot_ids, B.n_accept, B.extra_token,
                               D.batch, gamma, D.max_new, B.rs, out_ids, n_out, c->mirror_dev, c->st));
   return SDD_OK;
@@ -1035,12 +1034,8 @@ int32_t sdd_accept_logits(const float* logits_p, const float* logits_q, const in
   if (((uintptr_t)logits_p & 15u) || ((uintptr_t)logits_q & 15u) || ((uintptr_t)scratch & 15u)) return SDD_E_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   const float itp = temp_p > 0.f ? 1.f / temp_p : 0.f, itq = temp_q > 0.f ? 1.f / temp_q : 0.f;
-  float2* partial = (float2*)scratch;
-  const long long rows_p = (long long)rows * (gamma + 1), rows_q = (long long)rows * gamma;
-  const int chunks = stats_chunks_for(V);
-  SDD_CUDA(launch_row_stats(logits_p, rows_p, logits_q, itp == 0.f ? 0 : rows_q, V, itp, itq, partial, st));
-  SDD_CUDA(launch_accept(logits_p, logits_q, draft_ids, nullptr, nullptr, partial, chunks, partial + rows_p * chunks, chunks, rows, gamma, V, itp, itq,
-                         make_key(seed), (uint32_t)round, nullptr, accept_prob, n_accept, nullptr, out_ids, st));
+  SDD_CUDA(launch_accept_standalone(logits_p, logits_q, draft_ids, rows, gamma, V, itp, itq, make_key(seed), (uint32_t)round, n_accept, out_ids,
+                                    accept_prob, (float2*)scratch, st));
   return SDD_OK;
 }
 

@@ -56,10 +56,10 @@ __device__ __forceinline__ float scalar_uniform(PhiloxKey key, uint32_t purpose,
   return word_to_uniform(philox4x32_10(0u, j, rnd, rng_c3(purpose, k, b), key).x);
 }
 
-// Gumbel variate -log(-log u) for u = odd multiple of 2^-24 in (0, 1), to about 2e-6 absolute.
-// The inner logarithm needs care next to u = 1, where the largest variates (the likely arg-max winners) come
-// from: there 1 - u is exact in fp32 and -log(1 - t) is summed as a series; elsewhere the hardware log2 does.
-__device__ __forceinline__ float gumbel_from_uniform(float u) {
+// Exponential variate -log u for u = odd multiple of 2^-24 in (0, 1), to about 3e-6 relative.
+// The logarithm needs care next to u = 1, where the smallest variates (the likely winners of a race) come from: there
+// 1 - u is exact in fp32 and -log(1 - t) is summed as a series; elsewhere the hardware log2 does.
+__device__ __forceinline__ float exponential_from_uniform(float u) {
   const float t = 1.0f - u;
   float ser = fmaf(t, 1.f / 9.f, 1.f / 8.f);
   ser = fmaf(t, ser, 1.f / 7.f);
@@ -69,9 +69,10 @@ __device__ __forceinline__ float gumbel_from_uniform(float u) {
   ser = fmaf(t, ser, 1.f / 3.f);
   ser = fmaf(t, ser, 1.f / 2.f);
   ser = fmaf(t, ser, 1.f);
-  const float y = t < 0.125f ? t * ser : -__logf(u);
-  return -__logf(y);
+  return t < 0.125f ? t * ser : -__logf(u);
 }
+// Gumbel variate -log(-log u), to about 2e-6 absolute
+__device__ __forceinline__ float gumbel_from_uniform(float u) { return -__logf(exponential_from_uniform(u)); }
 
 // ---------------------------------------------------------------------------------------------
 // reductions

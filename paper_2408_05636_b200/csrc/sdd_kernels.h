@@ -64,13 +64,14 @@ cudaError_t launch_row_stats(const float* a, long long rows_a, const float* b, l
 cudaError_t launch_unmask_sample(const float* step_logits, int* slot_ids, float* q_logits, float* logq, float* lseq,
                                  int* reveal_step, int batch, int gamma, int V, int k, float inv_tau_q, PhiloxKey key,
                                  RoundState* rs, int cache_skip, cudaStream_t st);
-// round pipeline: logq_in / lseq_in from the draws, partial_q null; stand-alone: logq_in / lseq_in null, partial_q given
-// chunks_p / chunks_q: pairs per row in partial_p / partial_q
+// round pipeline: logq_in / lseq_in from the draws, chunks_p pairs per row in partial_p
 cudaError_t launch_accept(const float* logits_p, const float* q_rows, const int* draft_ids, const float* logq_in,
-                          const float* lseq_in, const float2* partial_p, int chunks_p, const float2* partial_q, int chunks_q,
-                          int rows, int gamma, int V,
-                          float inv_tau_p, float inv_tau_q_rows, PhiloxKey key, uint32_t rnd, RoundState* rs, float* accept_prob,
-                          int* n_accept, int* extra_token, int* out_ids, cudaStream_t st);
+                          const float* lseq_in, const float2* partial_p, int chunks_p, int rows, int gamma, int V, float inv_tau_p,
+                          PhiloxKey key, RoundState* rs, float* accept_prob, int* n_accept, int* extra_token, cudaStream_t st);
+// stand-alone; scratch: (rows * (2 gamma + 1)) * stats_chunks_for(V) pairs
+cudaError_t launch_accept_standalone(const float* logits_p, const float* logits_q, const int* draft_ids, int rows, int gamma, int V,
+                                     float inv_tau_p, float inv_tau_q, PhiloxKey key, uint32_t rnd, int* n_accept, int* out_ids,
+                                     float* accept_prob, float2* scratch, cudaStream_t st);
 cudaError_t launch_commit(int* tokens, int tok_stride, int* ctx_len, int* n_emitted, const int* slot_ids,
                           const int* n_accept, const int* extra_token, int batch, int gamma, int max_new, RoundState* rs,
                           int* out_ids, int* n_out, volatile int* host_mirror, cudaStream_t st);

@@ -216,19 +216,18 @@ constexpr int VC = 8;
 
 struct RowPartial {
   float arg_s; int arg_i;      // Gumbel arg-max of this CTA's share
-  float fb_s; int fb_i;        // fall-back arg-max (draw from p itself)
   float m, s;                  // online soft-max pair of this CTA's share
 };
 
-__device__ __forceinline__ ArgMax cluster_merge_argmax(cg::cluster_group& cl, RowPartial* mine, bool fallback) {
+__device__ __forceinline__ ArgMax cluster_merge_argmax(cg::cluster_group& cl, RowPartial* mine) {
   ArgMax a;
   a.s = -INFINITY;
   a.i = 0x7fffffff;
   for (int r = 0; r < VC; ++r) {
     const RowPartial* o = cl.map_shared_rank(mine, r);
     ArgMax b;
-    b.s = fallback ? o->fb_s : o->arg_s;
-    b.i = fallback ? o->fb_i : o->arg_i;
+    b.s = o->arg_s;
+    b.i = o->arg_i;
     a = argmax_better(a, b);
   }
   return a;
@@ -318,7 +317,7 @@ __device__ __forceinline__ void draw_slot(const float* src, float* __restrict__ 
   }
   cl.sync();
   if (rank == 0 && threadIdx.x == 0) {
-    ArgMax win = cluster_merge_argmax(cl, &part, false);
+    ArgMax win = cluster_merge_argmax(cl, &part);
     const float lse = greedy ? 0.f : cluster_merge_lse(cl, &part);
     if ((unsigned)win.i >= (unsigned)V) {   // no entry compared greater than -inf: the logits are not numbers
       win.i = 0;
@@ -398,42 +397,109 @@ ar_sample_kernel(const float* logits, int rows_per_seq, int* __restrict__ slot_i
 //
 // logits_p [rows, gamma+1, V]; q rows [rows, gamma, V] hold z_q = l * inv_tau_q_rows (inv_tau_q_rows
 // = 1 when the rows were stored already divided by the temperature).  log q(x) and the q rows' log-sum-exp come
-// either from `logq_in` / `lseq_in` (round pipeline: stored by the draw) or from the q-row partial statistics
+// either from `logq_in` / `lseq_in` (round pipeline: stored by the draw) or from the q-row statistics
 // (stand-alone call).  A draft id outside [0, V) is never used as an index: its row counts as rejected, the
 // sequence's n_accept becomes -1 (out_ids all -1) and, in the round pipeline, the status word DEV_BAD_TOKEN.
 // ---------------------------------------------------------------------------------------------
-constexpr int ACCEPT_THREADS = 256;
+struct AcceptArgs {
+  const float *logits_p, *q_rows;
+  const int* draft_ids;
+  const float *logq_in, *lseq_in;
+  int gamma, V;
+  float inv_tau_p, inv_tau_q;
+  PhiloxKey key;
+  uint32_t rnd;
+  RoundState* rs;
+  float* accept_prob;
+  int *n_accept, *extra_token, *out_ids;
+};
 
-// four CTAs per SM (64 registers): the stand-alone call's 8 x rows CTAs then fit in one wave for 64 rows
-__global__ void __cluster_dims__(VC, 1, 1) __launch_bounds__(ACCEPT_THREADS, 4)
-accept_kernel(const float* logits_p, const float* q_rows, const int* draft_ids,
-              const float* logq_in, const float* lseq_in, const float2* partial_p,
-              int chunks, const float2* partial_q, int chunks_q, int gamma, int V, float inv_tau_p,
-              float inv_tau_q_rows, PhiloxKey key, uint32_t rnd_arg, RoundState* __restrict__ rs,
-              float* __restrict__ accept_prob, int* __restrict__ n_accept, int* __restrict__ extra_token,
-              int* __restrict__ out_ids) {
+// Gumbel-max draw over a cluster's CTAs as a race of exponentials: arg-max of log w + G is arg-max of w / E with E = -log u, so
+// a token costs one logarithm and one reciprocal.  w = p (resid: max(0, p - q), tokens without mass never win).  The score
+// of the winner, 0 if no token had any mass.
+template <int THREADS>
+__device__ __forceinline__ ArgMax race_scan(const float* prow, const float* qrow, bool resid, float lsep, float lseq, const AcceptArgs& A,
+                                            uint32_t n, uint32_t rnd, uint32_t c3, int rank) {
+  constexpr float LOG2E = 1.4426950408889634f;
+  const float kp = A.inv_tau_p * LOG2E, kq = A.inv_tau_q * LOG2E, op = lsep * LOG2E, oq = lseq * LOG2E;
+  ArgMax best;
+  best.s = 0.f;
+  best.i = 0x7fffffff;
+  const int V = A.V, nblk = (V + 3) >> 2;
+  // two blocks of four entries per iteration, with all loads of the iteration issued before any arithmetic
+  constexpr int UNR = 2;
+  for (int blk0 = rank * THREADS + threadIdx.x; blk0 < nblk; blk0 += UNR * VC * THREADS) {
+    float xp[UNR][4], xq[UNR][4];
+#pragma unroll
+    for (int u = 0; u < UNR; ++u) {
+      const int v0 = (blk0 + u * VC * THREADS) * 4;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        xp[u][c] = v0 + c < V ? prow[v0 + c] : -INFINITY;
+        xq[u][c] = resid && v0 + c < V ? qrow[v0 + c] : -INFINITY;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < UNR; ++u) {
+      const int blk = blk0 + u * VC * THREADS;
+      if (blk >= nblk) break;
+      const uint4 w4 = philox4x32_10((uint32_t)blk, n, rnd, c3, A.key);
+      const uint32_t ww[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        float w = exp2f(fmaf(xp[u][c], kp, -op));
+        if (resid) w -= exp2f(fmaf(xq[u][c], kq, -oq));
+        const float sc = __fdividef(w, exponential_from_uniform(word_to_uniform(ww[c])));
+        if (sc > best.s) { best.s = sc; best.i = blk * 4 + c; }      // a thread's tokens come in ascending order
+      }
+    }
+  }
+  return best;
+}
+
+// The statistics come as pairs per row (row_stats_kernel, LM-head epilogue).  256 threads, four CTAs per SM (64 registers):
+// the stand-alone call's 8 x rows CTAs then fit in one wave for 64 rows.  1024 threads for a few rows: a row's chain (merge,
+// tests, scan of 50 k tokens) is what such a launch is bound by (1 x 5 x 50257, both launches: 16.0 -> 11.8 us); at 18 rows,
+// where CTAs of 1024 threads leave no room for the next sequences', 256 are better (27.3 against 21.2 us).
+template <int THREADS>
+__global__ void __cluster_dims__(VC, 1, 1) __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1)
+accept_kernel(AcceptArgs A, const float2* partial_p, int chunks, const float2* partial_q, int chunks_q) {
   pdl_launch_dependents();
   pdl_wait();
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank();
-  const int b = blockIdx.x / VC;
-  const uint32_t rnd = rs != nullptr ? rs->round : rnd_arg;
-  const bool greedy = inv_tau_p == 0.f;
+  const int b = blockIdx.x / VC, gamma = A.gamma, V = A.V;
+  if (A.rs != nullptr) A.rnd = A.rs->round;
+  const bool greedy = A.inv_tau_p == 0.f;
   extern __shared__ float s_dyn[];           // [gamma+1] lse_p (or arg-max bits), [gamma] lse_q
   float* s_lsep = s_dyn;
   float* s_lseq = s_dyn + gamma + 1;
   __shared__ int s_n, s_bad;
-  __shared__ int s_rej[ACCEPT_THREADS / 32];
-  __shared__ float s_val[ACCEPT_THREADS / 32];
-  __shared__ int s_idx[ACCEPT_THREADS / 32];
-  __shared__ RowPartial part;
-
+  __shared__ int s_rej[THREADS / 32];
+  __shared__ float s_val[THREADS / 32];
+  __shared__ int s_idx[THREADS / 32];
+  __shared__ ArgMax s_part[2][VC];           // the CTAs' winners, pushed into every CTA of the cluster (per pass)
   if (threadIdx.x == 0) s_bad = 0;
+
+  // the drafts' logits and uniforms (thread j: position j, gamma <= 256 <= THREADS), on their way while the pairs are merged
+  int draft = 0;
+  float xp = 0.f, xq = 0.f, uni = 0.f;
+  const bool tests = (int)threadIdx.x < gamma;
+  if (tests) {
+    const int j = threadIdx.x;
+    const long long jq = (long long)b * gamma + j;
+    draft = A.draft_ids[jq];
+    uni = scalar_uniform(A.key, RNG_ACCEPT, A.rnd, 0u, (uint32_t)j, (uint32_t)b);
+    if (!greedy && (unsigned)draft < (unsigned)V) {
+      xp = A.logits_p[((long long)b * (gamma + 1) + j) * V + draft];
+      xq = A.logq_in != nullptr ? A.logq_in[jq] : A.q_rows[jq * V + draft];
+    }
+  }
   const float2* pp = partial_p + (long long)b * (gamma + 1) * chunks;
   // the rows' pairs are merged by groups of lanes sized to the number of pairs (7 from row_stats_kernel: a thread per
   // row; 393 from the LM head's epilogue: a warp per row)
   {
-    const int tpr = merge_group_size(chunks), sub = (int)threadIdx.x % tpr, par = ACCEPT_THREADS / tpr;
+    const int tpr = merge_group_size(chunks), sub = (int)threadIdx.x % tpr, par = THREADS / tpr;
     for (int j0 = 0; j0 <= gamma; j0 += par) {
       const int j = j0 + (int)threadIdx.x / tpr;
       const bool valid = j <= gamma;
@@ -445,7 +511,7 @@ accept_kernel(const float* logits_p, const float* q_rows, const int* draft_ids,
   }
   if (partial_q != nullptr && !greedy) {
     const float2* pq = partial_q + (long long)b * gamma * chunks_q;
-    const int tpr = merge_group_size(chunks_q), sub = (int)threadIdx.x % tpr, par = ACCEPT_THREADS / tpr;
+    const int tpr = merge_group_size(chunks_q), sub = (int)threadIdx.x % tpr, par = THREADS / tpr;
     for (int j0 = 0; j0 < gamma; j0 += par) {
       const int j = j0 + (int)threadIdx.x / tpr;
       const bool valid = j < gamma;
@@ -455,132 +521,68 @@ accept_kernel(const float* logits_p, const float* q_rows, const int* draft_ids,
   }
   __syncthreads();
 
-  // first rejected position, computed identically by every CTA of the cluster (gamma <= ACCEPT_THREADS)
+  // first rejected position, computed identically by every CTA of the cluster
   int rej = gamma;
-  if ((int)threadIdx.x < gamma) {
+  if (tests) {
     const int j = threadIdx.x;
-    const int x = draft_ids[(long long)b * gamma + j];
     float ratio;
-    if ((unsigned)x >= (unsigned)V) {
+    if ((unsigned)draft >= (unsigned)V) {
       ratio = 0.f;
       s_bad = 1;
     } else if (greedy) {
-      ratio = (x == __float_as_int(s_lsep[j])) ? 1.f : 0.f;
+      ratio = (draft == __float_as_int(s_lsep[j])) ? 1.f : 0.f;
     } else {
-      const float logp = logits_p[((long long)b * (gamma + 1) + j) * V + x] * inv_tau_p - s_lsep[j];
-      const float lq = logq_in != nullptr ? logq_in[(long long)b * gamma + j]
-                                          : q_rows[((long long)b * gamma + j) * V + x] * inv_tau_q_rows - s_lseq[j];
-      ratio = expf(fminf(0.f, logp - lq));
+      const float lq = A.logq_in != nullptr ? xq : xq * A.inv_tau_q - s_lseq[j];
+      ratio = expf(fminf(0.f, xp * A.inv_tau_p - s_lsep[j] - lq));
     }
-    const float u = scalar_uniform(key, RNG_ACCEPT, rnd, 0u, (uint32_t)j, (uint32_t)b);
-    if (rank == 0) accept_prob[(long long)b * gamma + j] = ratio;
-    if (!(u <= ratio)) rej = j;
+    if (rank == 0) A.accept_prob[(long long)b * gamma + j] = ratio;
+    if (!(uni <= ratio)) rej = j;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) rej = min(rej, __shfl_xor_sync(0xffffffffu, rej, o));
   if ((threadIdx.x & 31) == 0) s_rej[threadIdx.x >> 5] = rej;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int n = gamma;
-    for (int w = 0; w < ACCEPT_THREADS / 32; ++w) n = min(n, s_rej[w]);
-    s_n = n;
-  }
-  __syncthreads();
-  const int n = s_n;
+  int n = gamma;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) n = min(n, s_rej[w]);      // gamma <= 256: the tests are the first eight warps'
 
   // extra token: residual of row n (n < gamma) or the bonus draw from row gamma
-  const float* prow = logits_p + ((long long)b * (gamma + 1) + n) * V;
   const bool resid = n < gamma;
-  ArgMax best, fallback;
-  best.s = -INFINITY;
-  best.i = 0x7fffffff;
-  fallback = best;
-  if (!greedy) {
-    const float* qrow = q_rows + ((long long)b * gamma + (resid ? n : 0)) * V;
-    const float lsep = s_lsep[n];
-    float lseq = 0.f;
-    if (resid) {
-      // stand-alone call: from the q rows' chunk statistics; round pipeline: stored by the draw of slot n
-      lseq = partial_q != nullptr ? s_lseq[n] : lseq_in[(long long)b * gamma + n];
+  const float* prow = A.logits_p + ((long long)b * (gamma + 1) + n) * V;
+  const float* qrow = A.q_rows + ((long long)b * gamma + (resid ? n : 0)) * V;
+  const float lseq = !resid || greedy ? 0.f : partial_q != nullptr ? s_lseq[n] : A.lseq_in[(long long)b * gamma + n];
+  const uint32_t c3 = rng_c3(resid ? RNG_RESID : RNG_BONUS, 0u, (uint32_t)b);
+  int t = greedy ? __float_as_int(s_lsep[n]) : 0;     // greedy: arg-max of the target row, in both branches
+  // pass 1, in all but degenerate cases never entered: max(0, p - q) has no mass anywhere, the draw is from p itself
+  for (int pass = 0; pass < 2 && !greedy; ++pass) {
+    ArgMax best = race_scan<THREADS>(prow, qrow, resid && pass == 0, s_lsep[n], lseq, A, (uint32_t)n, A.rnd, c3, rank);
+    best = block_argmax<THREADS>(best, s_val, s_idx);
+    if (threadIdx.x < 32) {
+      best.s = __shfl_sync(0xffffffffu, best.s, 0);
+      best.i = __shfl_sync(0xffffffffu, best.i, 0);
+      if (threadIdx.x < VC) *cl.map_shared_rank(&s_part[pass][rank], (int)threadIdx.x) = best;
     }
-    const uint32_t c3 = rng_c3(resid ? RNG_RESID : RNG_BONUS, 0u, (uint32_t)b);
-    const int nblk = (V + 3) >> 2;
-    // two blocks of four entries per iteration, with all loads of the iteration issued before any arithmetic
-    constexpr int UNR = 2;
-    for (int blk0 = rank * ACCEPT_THREADS + threadIdx.x; blk0 < nblk; blk0 += UNR * VC * ACCEPT_THREADS) {
-      float xp[UNR][4], xq[UNR][4];
+    cl.sync();     // every CTA has everybody's winner: all of them have to know whether the second pass is needed
+    ArgMax win = s_part[pass][0];
 #pragma unroll
-      for (int u = 0; u < UNR; ++u) {
-        const int blk = blk0 + u * VC * ACCEPT_THREADS;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int v = blk * 4 + c;
-          const bool in = blk < nblk && v < V;
-          xp[u][c] = in ? __ldg(prow + v) : 0.f;
-          xq[u][c] = (in && resid) ? __ldg(qrow + v) : 0.f;
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < UNR; ++u) {
-        const int blk = blk0 + u * VC * ACCEPT_THREADS;
-        if (blk >= nblk) break;
-        const uint4 w = philox4x32_10((uint32_t)blk, (uint32_t)n, rnd, c3, key);
-        const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int v = blk * 4 + c;
-          if (v < V) {
-            const float g = gumbel_from_uniform(word_to_uniform(ww[c]));
-            const float zp = xp[u][c] * inv_tau_p - lsep;   // log p_v
-            ArgMax cand;
-            cand.i = v;
-            cand.s = zp + g;
-            if (resid) {
-              fallback = argmax_better(fallback, cand);    // a draw from p itself, if max(0, p - q) == 0 everywhere
-              const float zq = xq[u][c] * inv_tau_q_rows - lseq;
-              const float wv = __expf(zp) - __expf(zq);
-              if (wv > 0.f) {
-                cand.s = __logf(wv) + g;
-                best = argmax_better(best, cand);
-              }
-            } else {
-              best = argmax_better(best, cand);
-            }
-          }
-        }
-      }
-    }
-    best = block_argmax<ACCEPT_THREADS>(best, s_val, s_idx);
-    __syncthreads();
-    fallback = block_argmax<ACCEPT_THREADS>(fallback, s_val, s_idx);
+    for (int w = 1; w < VC; ++w) win = argmax_better(win, s_part[pass][w]);
+    t = win.i;
+    if (t != 0x7fffffff || !resid) break;
+  }
+  if (rank != 0 || threadIdx.x >= 32) return;
+  bool bad = s_bad != 0;
+  if ((unsigned)t >= (unsigned)V) {   // no entry compared greater than nothing: the logits are not numbers
+    t = 0;
+    bad = true;
   }
   if (threadIdx.x == 0) {
-    part.arg_s = best.s; part.arg_i = best.i; part.fb_s = fallback.s; part.fb_i = fallback.i;
+    if (bad && A.rs != nullptr) atomicCAS(&A.rs->status, DEV_OK, DEV_BAD_TOKEN);
+    A.n_accept[b] = bad ? -1 : n;
+    if (A.extra_token != nullptr) A.extra_token[b] = t;
   }
-  cl.sync();
-  if (rank == 0 && threadIdx.x == 0) {
-    int t;
-    if (greedy) {
-      t = __float_as_int(s_lsep[n]);   // arg-max of the target row, in both branches
-    } else {
-      ArgMax win = cluster_merge_argmax(cl, &part, false);
-      if (win.i == 0x7fffffff) win = cluster_merge_argmax(cl, &part, true);
-      t = win.i;
-    }
-    bool bad = s_bad != 0;
-    if ((unsigned)t >= (unsigned)V) {   // no entry compared greater than -inf: the logits are not numbers
-      t = 0;
-      bad = true;
-    }
-    if (bad && rs != nullptr) atomicCAS(&rs->status, DEV_OK, DEV_BAD_TOKEN);
-    n_accept[b] = bad ? -1 : n;
-    if (extra_token != nullptr) extra_token[b] = t;
-    if (out_ids != nullptr) {
-      for (int j = 0; j <= gamma; ++j)
-        out_ids[(long long)b * (gamma + 1) + j] = bad ? -1 : (j < n ? draft_ids[(long long)b * gamma + j] : (j == n ? t : -1));
-    }
-  }
-  cl.sync();   // partials stay alive until rank 0 has read them
+  if (A.out_ids != nullptr)
+    for (int j = threadIdx.x; j <= gamma; j += 32)
+      A.out_ids[(long long)b * (gamma + 1) + j] = bad ? -1 : (j < n ? A.draft_ids[(long long)b * gamma + j] : (j == n ? t : -1));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -684,16 +686,33 @@ cudaError_t launch_ar_sample(const float* logits, int rows_per_seq, int* slot_id
   return cudaGetLastError();
 }
 
+static cudaError_t launch_accept_args(const AcceptArgs& A, const float2* partial_p, int chunks_p, const float2* partial_q, int chunks_q,
+                                      int rows, cudaStream_t st) {
+  const size_t smem = (size_t)(2 * A.gamma + 1) * sizeof(float);
+  if (rows <= 8)
+    return launch_k(accept_kernel<1024>, dim3(VC * rows), dim3(1024), smem, st, A, partial_p, chunks_p, partial_q, chunks_q);
+  return launch_k(accept_kernel<256>, dim3(VC * rows), dim3(256), smem, st, A, partial_p, chunks_p, partial_q, chunks_q);
+}
+
 cudaError_t launch_accept(const float* logits_p, const float* q_rows, const int* draft_ids, const float* logq_in,
-                          const float* lseq_in, const float2* partial_p, int chunks_p, const float2* partial_q, int chunks_q,
-                          int rows, int gamma, int V,
-                          float inv_tau_p, float inv_tau_q_rows, PhiloxKey key, uint32_t rnd, RoundState* rs, float* accept_prob,
-                          int* n_accept, int* extra_token, int* out_ids, cudaStream_t st) {
-  const size_t smem = (size_t)(2 * gamma + 1) * sizeof(float);
-  launch_k(accept_kernel, dim3(VC * rows), dim3(ACCEPT_THREADS), smem, st, logits_p, q_rows, draft_ids, logq_in, lseq_in, partial_p,
-                                                    chunks_p, partial_q, chunks_q, gamma, V, inv_tau_p, inv_tau_q_rows, key, rnd, rs,
-                                                    accept_prob, n_accept, extra_token, out_ids);
-  return cudaGetLastError();
+                          const float* lseq_in, const float2* partial_p, int chunks_p, int rows, int gamma, int V, float inv_tau_p,
+                          PhiloxKey key, RoundState* rs, float* accept_prob, int* n_accept, int* extra_token, cudaStream_t st) {
+  const AcceptArgs A = {logits_p, q_rows, draft_ids, logq_in, lseq_in, gamma, V, inv_tau_p, inv_tau_p == 0.f ? 0.f : 1.f, key, 0u, rs,
+                        accept_prob, n_accept, extra_token, nullptr};
+  return launch_accept_args(A, partial_p, chunks_p, nullptr, 0, rows, st);
+}
+
+cudaError_t launch_accept_standalone(const float* logits_p, const float* logits_q, const int* draft_ids, int rows, int gamma, int V,
+                                     float inv_tau_p, float inv_tau_q, PhiloxKey key, uint32_t rnd, int* n_accept, int* out_ids,
+                                     float* accept_prob, float2* scratch, cudaStream_t st) {
+  const AcceptArgs A = {logits_p, logits_q, draft_ids, nullptr, nullptr, gamma, V, inv_tau_p, inv_tau_q, key, rnd, nullptr,
+                        accept_prob, n_accept, nullptr, out_ids};
+  const bool greedy = inv_tau_p == 0.f;
+  const long long rows_p = (long long)rows * (gamma + 1), rows_q = (long long)rows * gamma;
+  const int chunks = stats_chunks(V);
+  cudaError_t e = launch_row_stats(logits_p, rows_p, logits_q, greedy ? 0 : rows_q, V, inv_tau_p, inv_tau_q, scratch, st);
+  if (e != cudaSuccess) return e;
+  return launch_accept_args(A, scratch, chunks, scratch + rows_p * chunks, chunks, rows, st);
 }
 
 cudaError_t launch_commit(int* tokens, int tok_stride, int* ctx_len, int* n_emitted, const int* slot_ids,
