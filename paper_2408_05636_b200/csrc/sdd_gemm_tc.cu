@@ -91,6 +91,15 @@ __device__ __forceinline__ void stage_bias(float* bias_s, const float* __restric
   stage_bias(bias_s, bias, n0, rows_b, whole_tile_group<BN>());
 }
 
+// eight accumulator columns plus their bias values, as four pairs (bias_s: 16-byte aligned shared memory)
+__device__ __forceinline__ void biased8(const uint32_t* v, const float* bias_s, uint64_t (&x)[4]) {
+  const float4 b0 = *reinterpret_cast<const float4*>(bias_s), b1 = *reinterpret_cast<const float4*>(bias_s + 4);
+  x[0] = f2_add(f2_pack(__uint_as_float(v[0]), __uint_as_float(v[1])), f2_pack(b0.x, b0.y));
+  x[1] = f2_add(f2_pack(__uint_as_float(v[2]), __uint_as_float(v[3])), f2_pack(b0.z, b0.w));
+  x[2] = f2_add(f2_pack(__uint_as_float(v[4]), __uint_as_float(v[5])), f2_pack(b1.x, b1.y));
+  x[3] = f2_add(f2_pack(__uint_as_float(v[6]), __uint_as_float(v[7])), f2_pack(b1.z, b1.w));
+}
+
 template <int BN>
 __device__ __forceinline__ void epilogue_tma(uint32_t tmem_acc, int m0, int n0, int q, int lane, int epi,
                                              const float* bias_s, const CUtensorMap* map_out,
@@ -132,29 +141,23 @@ __device__ __forceinline__ void epilogue_tma(uint32_t tmem_acc, int m0, int n0, 
     uint8_t* row = stage_generic + buf * (128 * 128) + rl * 128;
     if (f32) {
 #pragma unroll
-      for (int g = 0; g < 8; ++g) {
-        float4 x;
-        x.x = __uint_as_float(v[g * 4 + 0]) + bias_s[cc * 32 + g * 4 + 0];
-        x.y = __uint_as_float(v[g * 4 + 1]) + bias_s[cc * 32 + g * 4 + 1];
-        x.z = __uint_as_float(v[g * 4 + 2]) + bias_s[cc * 32 + g * 4 + 2];
-        x.w = __uint_as_float(v[g * 4 + 3]) + bias_s[cc * 32 + g * 4 + 3];
-        *reinterpret_cast<float4*>(row + ((g ^ sw) << 4)) = x;
+      for (int g = 0; g < 4; ++g) {
+        uint64_t x[4];
+        biased8(v + g * 8, bias_s + cc * 32 + g * 8, x);
+        *reinterpret_cast<ulonglong2*>(row + (((2 * g) ^ sw) << 4)) = make_ulonglong2(x[0], x[1]);
+        *reinterpret_cast<ulonglong2*>(row + (((2 * g + 1) ^ sw) << 4)) = make_ulonglong2(x[2], x[3]);
       }
     } else {
 #pragma unroll
       for (int g = 0; g < 4; ++g) {
-        uint32_t pk[4];
+        uint64_t x[4];
+        biased8(v + g * 8, bias_s + cc * 32 + g * 8, x);
+        if (epi == EPI_GELU) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int j0 = g * 8 + 2 * e;
-          float x0 = __uint_as_float(v[j0]) + bias_s[cc * 32 + j0];
-          float x1 = __uint_as_float(v[j0 + 1]) + bias_s[cc * 32 + j0 + 1];
-          if (epi == EPI_GELU) { x0 = gelu_tanh_fast(x0); x1 = gelu_tanh_fast(x1); }
-          __nv_bfloat162 h2 = __floats2bfloat162_rn(x0, x1);
-          pk[e] = *reinterpret_cast<uint32_t*>(&h2);
+          for (int e = 0; e < 4; ++e) x[e] = f2_gelu(x[e]);
         }
         const int chunk = (cc & 1) * 4 + g;
-        *reinterpret_cast<uint4*>(row + ((chunk ^ sw) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        *reinterpret_cast<uint4*>(row + ((chunk ^ sw) << 4)) = make_uint4(f2_bf16(x[0]), f2_bf16(x[1]), f2_bf16(x[2]), f2_bf16(x[3]));
       }
     }
     if (last_of_buf) {
@@ -206,25 +209,22 @@ __device__ __forceinline__ void epilogue_qkv(uint32_t tmem_acc, int m0, int n0, 
     uint8_t* bp = stage_generic + buf * (128 * 128);
     if (is_v) {
       bp += box_off;
+      float bv[32];
+#pragma unroll
+      for (int g = 0; g < 8; ++g) *reinterpret_cast<float4*>(bv + 4 * g) = *reinterpret_cast<const float4*>(bias_s + cc * 32 + 4 * g);
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
         const int jj = (cc & 1) * 32 + j;      // feature row inside the buffer
-        const float x = __uint_as_float(v[j]) + bias_s[cc * 32 + j];
+        const float x = __uint_as_float(v[j]) + bv[j];
         *reinterpret_cast<__nv_bfloat16*>(bp + jj * 128 + ((pchunk ^ (uint32_t)(jj & 7)) << 4) + in_row) = __float2bfloat16_rn(x);
       }
     } else {
       uint8_t* row = bp + rl * 128;
 #pragma unroll
       for (int g = 0; g < 4; ++g) {
-        uint32_t pk[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int j0 = g * 8 + 2 * e;
-          __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(v[j0]) + bias_s[cc * 32 + j0],
-                                                    __uint_as_float(v[j0 + 1]) + bias_s[cc * 32 + j0 + 1]);
-          pk[e] = *reinterpret_cast<uint32_t*>(&h2);
-        }
-        *reinterpret_cast<uint4*>(row + ((((cc & 1) * 4 + g) ^ sw) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        uint64_t x[4];
+        biased8(v + g * 8, bias_s + cc * 32 + g * 8, x);
+        *reinterpret_cast<uint4*>(row + ((((cc & 1) * 4 + g) ^ sw) << 4)) = make_uint4(f2_bf16(x[0]), f2_bf16(x[1]), f2_bf16(x[2]), f2_bf16(x[3]));
       }
     }
     if ((cc & 1) == 1) {
@@ -272,18 +272,14 @@ __device__ __forceinline__ void epilogue_pair_out(uint32_t tmem_acc, int m0, int
     uint8_t* row = stage_generic + buf * (128 * 128) + rl * 128;
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
+      uint64_t x[4];
       uint32_t pk[4];
+      biased8(v + g * 8, bias_s + cc * 32 + g * 8, x);
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const int j0 = g * 8 + 2 * e;
-        float x0 = __uint_as_float(v[j0]) + bias_s[cc * 32 + j0], x1 = __uint_as_float(v[j0 + 1]) + bias_s[cc * 32 + j0 + 1];
-        if (epi == EPI_GELU) { x0 = gelu_tanh_fast(x0); x1 = gelu_tanh_fast(x1); }
-        __nv_bfloat162 h2 = __floats2bfloat162_rn(x0, x1);
-        if (lo) {
-          const uint32_t hb = *reinterpret_cast<uint32_t*>(&h2);
-          h2 = __floats2bfloat162_rn(x0 - __uint_as_float(hb << 16), x1 - __uint_as_float(hb & 0xffff0000u));
-        }
-        pk[e] = *reinterpret_cast<uint32_t*>(&h2);
+        if (epi == EPI_GELU) x[e] = f2_gelu(x[e]);
+        pk[e] = f2_bf16(x[e]);
+        if (lo) pk[e] = f2_bf16(f2_add(x[e], f2_pack(-__uint_as_float(pk[e] << 16), -__uint_as_float(pk[e] & 0xffff0000u))));
       }
       *reinterpret_cast<uint4*>(row + ((((cc & 1) * 4 + g) ^ sw) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
     }

@@ -245,6 +245,46 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t cols)
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
 }
 
+// ---- packed pairs of fp32 (sm_100a issues one instruction for two operations) -----------------
+__device__ __forceinline__ uint64_t f2_pack(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint32_t f2_bf16(uint64_t v) {      // packed bf16x2, low half = first
+  float a, b;
+  f2_unpack(v, a, b);
+  __nv_bfloat162 t = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<uint32_t*>(&t);
+}
+// tanh-GELU of a pair with the hardware tanh (see gelu_tanh_fast): x/2 + x/2 tanh(x (c + 0.044715 c x^2))
+__device__ __forceinline__ uint64_t f2_gelu(uint64_t x) {
+  const float c = 0.7978845608028654f;
+  const uint64_t w = f2_mul(x, f2_fma(f2_mul(x, x), f2_pack(0.044715f * c, 0.044715f * c), f2_pack(c, c)));
+  float a, b;
+  f2_unpack(w, a, b);
+  asm("tanh.approx.f32 %0, %0;" : "+f"(a));
+  asm("tanh.approx.f32 %0, %0;" : "+f"(b));
+  const uint64_t h = f2_mul(x, f2_pack(0.5f, 0.5f));
+  return f2_fma(h, f2_pack(a, b), h);
+}
+
 // make generic-proxy writes to shared memory visible to the async proxy (TMA / tensor core reads)
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
