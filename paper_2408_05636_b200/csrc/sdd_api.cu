@@ -1,6 +1,7 @@
 // C ABI of the SpecDiff round: argument checking, workspace layout, and the host-side schedule
 // that enqueues the kernels of Algorithm 1 on the caller's stream.  See include/sdd.h.
 #include <atomic>
+#include <climits>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -190,7 +191,7 @@ struct sdd_ctx {
   bool hilo;                   // SDD_HILO != 0 (default): hi/lo activation pairs in the target's MLP and LM head
   bool force_simt;             // SDD_GEMM=simt: run bf16 GEMMs on the CUDA-core kernel (cross-check)
   int bn_hint;                 // SDD_GEMM_BN: N tile of the tensor-core GEMM (0 = choose)
-  int few_rows;                // SDD_FEW_ROWS (default 32): causal forwards of at most this many rows run on the weight-streaming kernels
+  int few_rows;                // SDD_FEW_ROWS (default: no limit of its own): causal forwards of at most this many rows run on the weight-streaming kernels
   bool head_stats;             // SDD_HEAD_STATS != 0 (default): soft-max statistics from the target LM head's epilogue
   bool use_graph;              // SDD_GRAPH != 0: sdd_step replays a captured graph per row-count bucket
   struct GraphEntry { cudaGraphExec_t exec; uint64_t launches; };
@@ -288,6 +289,11 @@ static int gemm(sdd_ctx* c, int cat, const void* A, size_t a_elems, const void* 
 template <typename T>
 static bool use_tc(const sdd_ctx* c, const Net& N) {
   return std::is_same<T, __nv_bfloat16>::value && !c->force_simt && N.d_head == 64;
+}
+
+// verification-like forwards of network N whose `rows` rows run on the weight-streaming kernels (run_blocks_few)
+static bool runs_few(const sdd_ctx* c, const Net& N, long long rows) {
+  return N.dtype == SDD_BF16 && !c->force_simt && N.d_head == 64 && rows <= c->few_rows && few_rows_fit((int)rows, N.d, N.d_head);
 }
 
 #define SDD_LAUNCH(c, cat, expr) \
@@ -446,7 +452,7 @@ static int forward_causal(sdd_ctx* c, const Net& N, void* kv, const int* len, in
   hilo = hilo && tc;
   // tensor-core path: per layer the cache is K [B][n_ctx][d] followed by V^T [B][d][n_ctx];
   // CUDA-core path: [B][n_ctx][K|V][d]
-  if (tc && mode == TARGET_VERIFY && rows <= c->few_rows && few_rows_fit((int)rows, N.d, N.d_head))
+  if (mode == TARGET_VERIFY && runs_few(c, N, rows))
     SDD_TRY(run_blocks_few(c, N, kv, len, rows_per_seq, hilo, gcat, acat));
   else
   SDD_TRY((run_blocks<T>(c, N, rows, gcat, hilo, nullptr,
@@ -676,7 +682,7 @@ int32_t sdd_create(const sdd_model* target, const sdd_model* drafter, const sdd_
     const char* hs = getenv("SDD_HEAD_STATS");
     c->head_stats = hs == nullptr || atoi(hs) != 0;
     const char* fr = getenv("SDD_FEW_ROWS");
-    c->few_rows = fr == nullptr ? 32 : atoi(fr);
+    c->few_rows = fr == nullptr ? INT_MAX : atoi(fr);
     const char* gr = getenv("SDD_GRAPH");
     // the legacy default stream cannot be captured: rounds are then enqueued kernel by kernel
     c->use_graph = (gr == nullptr || atoi(gr) != 0) && c->st != nullptr && c->st != cudaStreamLegacy;
@@ -832,7 +838,9 @@ int32_t sdd_step(sdd_ctx* c, int32_t* out_ids, int32_t* n_out) {
   SDD_TRY(round_prologue(c));
   // per-launch timing: the event pairs are captured into a one-off graph, so the stamps are taken on the device
   // timeline without host launch gaps in between
-  const int few = attn_few_fits(c->D.gamma + 1, c->P.n_ctx) ? c->key_splits : 0;
+  const int R = c->D.gamma + 1;
+  const int few = runs_few(c, c->P, (long long)c->D.batch * R) && attn_few_fits(R, c->P.n_ctx)
+                      ? attn_few_splits(c->D.batch, R, c->P.n_head, c->key_splits) : 0;
   const auto key = std::make_tuple(c->profiling ? -c->lcap - (int)c->prof_graphs.size() - 1 : c->lcap + few, (void*)out_ids,
                                    (void*)n_out);
   auto it = c->graphs.find(key);

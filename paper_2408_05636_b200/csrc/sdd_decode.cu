@@ -274,7 +274,7 @@ gemv_add_kernel(const __nv_bfloat16* xin, const __nv_bfloat16* xin_lo, const __n
 enum StreamOut : int { SO_ADD = 0, SO_GELU = 1, SO_QKV = 2 };
 
 template <int MT, int CG, bool LO>
-__global__ void __launch_bounds__(THREADS, MT == 1 && CG <= 2 ? 3 : MT <= 2 && CG <= 4 ? 2 : 1)
+__global__ void __launch_bounds__(THREADS, MT == 1 && CG <= 2 ? 3 : MT <= 2 && CG <= 5 ? 2 : 1)
 stream_kernel(const __nv_bfloat16* x, const __nv_bfloat16* x_lo, const __nv_bfloat16* __restrict__ W, const float* __restrict__ bias, int M,
               int K, int N, int kind, void* out, __nv_bfloat16* out_lo, const QkvDst qd, int* status) {
   constexpr int R = 16 * MT, C = 8 * CG, TILE = R * C;
@@ -308,7 +308,7 @@ stream_kernel(const __nv_bfloat16* x, const __nv_bfloat16* x_lo, const __nv_bflo
     }
   };
   // slices whose activations are in flight together (more of them spill: 8 at one column group cost 0.1 ms of a 1.2 ms step)
-  constexpr int NB = CG == 1 ? 4 : CG == 2 ? (LO ? 2 : 4) : 2;
+  constexpr int NB = MT == 3 ? (CG <= 4 ? 3 : CG <= 6 ? 2 : 1) : CG == 1 ? 4 : CG == 2 ? (LO ? 2 : 4) : CG <= 4 ? 2 : 1;
   bool ok = true, waited = false;
   for (int i0 = warp; i0 < n_sl; i0 += WARPS * NB) {
     uint4 hi[NB][CG], lo[LO ? NB : 1][LO ? CG : 1];
@@ -366,7 +366,9 @@ stream_kernel(const __nv_bfloat16* x, const __nv_bfloat16* x_lo, const __nv_bflo
 }
 
 // ---------------------------------------------------------------------------------------------
-// attention of R <= 8 new rows of a sequence (positions ctx_len - 1 + r) over its KV cache.  The keys of a head are dealt
+// attention of R new rows of a sequence (positions ctx_len - 1 + r) over its KV cache, eight rows to a CTA; what further groups
+// of rows read of the cache comes from L2 (33 rows of 25 heads, 512 keys: XL verification 2.99 -> 2.94 ms against one 128-row
+// tcgen05 CTA a head that walks all keys; 9 rows 1.99 -> 1.86).  The keys of a head are dealt
 // out in slices of 32 to a cluster of one, two or four CTAs (slice s to CTA s % S): what bounds the kernel is how fast an SM
 // takes in its part of the cache (one CTA per head: 4.5 us at 512 keys), so the heads are spread over the chip.
 // Scores are K (16 keys x 64) times Q^T (64 x 8 rows), the output V^T (16 features x keys) times P^T: both operands of both
@@ -380,21 +382,22 @@ struct FewParams {
   const __nv_bfloat16 *kc, *vt;
   __nv_bfloat16* out;
   const int* ctx_len;
-  int q_ld, R, n_ctx, d, s_ld, splits;
+  int q_ld, R, n_ctx, d, s_ld, splits, groups;
 };
 
 template <int R_MAX>
 __global__ void __launch_bounds__(32 * AT_WARPS, 2)
 attn_few_kernel(const FewParams p) {
   extern __shared__ __align__(128) uint8_t dyn[];
-  const int R = p.R, n_ctx = p.n_ctx, d = p.d, S = p.splits;
+  const int n_ctx = p.n_ctx, d = p.d, S = p.splits;
+  const int b = blockIdx.y / p.groups, r0 = (blockIdx.y - b * p.groups) * TOK, R = min(p.R - r0, R_MAX);     // rows r0 .. r0 + R - 1
   float* s_s = reinterpret_cast<float*>(dyn);                                 // [R][s_ld] scores of this CTA's keys
   __nv_bfloat16* s_p = reinterpret_cast<__nv_bfloat16*>(s_s + R * p.s_ld);    // [R][s_ld + 8] probabilities
   __shared__ float o_s[2][64][TOK];
   __shared__ float recv_o[4][64][R_MAX], recv_m[4][R_MAX], recv_l[4][R_MAX];  // partial states of the cluster's CTAs
   __shared__ float m_s[AT_WARPS], sum_s[AT_WARPS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int hd = blockIdx.x / S, rank = blockIdx.x % S, b = blockIdx.y;
+  const int hd = blockIdx.x / S, rank = blockIdx.x % S;
   const __nv_bfloat16* kb = p.kc + (long long)b * n_ctx * d + hd * 64;
   const __nv_bfloat16* vh = p.vt + ((long long)b * d + hd * 64) * n_ctx;
   {
@@ -408,12 +411,13 @@ attn_few_kernel(const FewParams p) {
   }
   pdl_launch_dependents();
   pdl_wait();
-  const int c = p.ctx_len[b];
+  const int c = p.ctx_len[b] + r0;                      // the first row's keys
   const int n_keys = min(c - 1 + R, n_ctx);
+  const long long row0 = (long long)b * p.R + r0;
   uint4 qf[2];
 #pragma unroll
   for (int i = 0; i < 2; ++i)
-    qf[i] = g < R ? *reinterpret_cast<const uint4*>(p.q + ((long long)b * R + g) * p.q_ld + hd * 64 + i * 32 + t * 8) : make_uint4(0, 0, 0, 0);
+    qf[i] = g < R ? *reinterpret_cast<const uint4*>(p.q + (row0 + g) * p.q_ld + hd * 64 + i * 32 + t * 8) : make_uint4(0, 0, 0, 0);
   const float scale = 0.125f * 1.4426950408889634f;                           // 1 / sqrt(64) * log2(e)
   // j: the CTA's 16-key tiles, two to a slice; slice i of the CTA is slice rank + S i of the sequence
   auto key_of = [&](int j) { return ((rank + S * (j >> 1)) * 2 + (j & 1)) * 16; };
@@ -542,7 +546,7 @@ attn_few_kernel(const FewParams p) {
       l = fmaf(recv_l[w][r], e, l);
       x = fmaf(recv_o[w][f][r], e, x);
     }
-    p.out[((long long)b * R + r) * d + hd * 64 + f] = __float2bfloat16_rn(x / l);
+    p.out[(row0 + r) * d + hd * 64 + f] = __float2bfloat16_rn(x / l);
   }
 }
 
@@ -577,6 +581,13 @@ cudaError_t prepare_decode() {
     set2(stream_kernel<1, 2, false>, stream_kernel<1, 2, true>);
     set2(stream_kernel<2, 3, false>, stream_kernel<2, 3, true>);
     set2(stream_kernel<2, 4, false>, stream_kernel<2, 4, true>);
+    set2(stream_kernel<2, 5, false>, stream_kernel<2, 5, true>);
+    set2(stream_kernel<2, 6, false>, stream_kernel<2, 6, true>);
+    set2(stream_kernel<2, 8, false>, stream_kernel<2, 8, true>);
+    set2(stream_kernel<3, 3, false>, stream_kernel<3, 3, true>);
+    set2(stream_kernel<3, 4, false>, stream_kernel<3, 4, true>);
+    set2(stream_kernel<3, 5, false>, stream_kernel<3, 5, true>);
+    set2(stream_kernel<3, 6, false>, stream_kernel<3, 6, true>);
     set(attn_few_kernel<1>, ATTN_SMEM_MAX);
     set(attn_few_kernel<2>, ATTN_SMEM_MAX);
     set(attn_few_kernel<8>, ATTN_SMEM_MAX);
@@ -584,8 +595,21 @@ cudaError_t prepare_decode() {
   return prep;
 }
 
-bool few_rows_fit(int M, int d, int d_head) { return M <= 32 && d_head == 64 && d <= 2048; }
-bool attn_few_fits(int R, int n_ctx) { return R <= dec::TOK && (n_ctx & 7) == 0 && dec::attn_smem(R, n_ctx, 1) <= dec::ATTN_SMEM_MAX; }
+// Up to 64 rows while FC1 is one wave of 32-feature CTAs (width 1184), up to 48 beyond: there every CTA's own copy of the
+// activations outweighs the weights' head start.  Against the tcgen05 kernels, 512 keys: 12 layers of width 768, 33 rows
+// 0.70 -> 0.52 ms, 64 rows 0.89 -> 0.65; 24 of 1024, 64 rows 1.73 -> 1.36; 48 of 1600, 33 rows 3.22 -> 2.94, 48 rows
+// 3.55 -> 3.40, but 49 rows 3.56 -> 3.86.
+bool few_rows_fit(int M, int d, int d_head) {
+  const bool one_wave = (4 * d + 31) / 32 <= dec::SMS;
+  return M <= (one_wave ? 64 : 48) && d_head == 64 && d <= 2048;
+}
+// CTAs that share a head's keys: `key_splits` (by the context's length) while that is no more than one CTA an SM
+int attn_few_splits(int batch, int R, int n_head, int key_splits) {
+  const int groups = (R + dec::TOK - 1) / dec::TOK;
+  while (key_splits > 1 && n_head * batch * groups * key_splits > dec::SMS) key_splits >>= 1;
+  return key_splits;
+}
+bool attn_few_fits(int R, int n_ctx) { return (n_ctx & 7) == 0 && dec::attn_smem(R < dec::TOK ? R : dec::TOK, n_ctx, 1) <= dec::ATTN_SMEM_MAX; }
 
 cudaError_t launch_gemv_ln(const float* h, const float* ln_g, const float* ln_b, const __nv_bfloat16* W, const float* bias, int M, int K,
                            int N, __nv_bfloat16* out, __nv_bfloat16* out_lo, const QkvDst* qkv, int* status, cudaStream_t st) {
@@ -602,7 +626,7 @@ cudaError_t launch_gemv_ln(const float* h, const float* ln_g, const float* ln_b,
 cudaError_t launch_stream_gemm(const __nv_bfloat16* x, const __nv_bfloat16* x_lo, const __nv_bfloat16* W, const float* bias, int M, int K, int N,
                                int epi, void* out, __nv_bfloat16* out_lo, const QkvDst* qkv, int* status, cudaStream_t st) {
   using namespace dec;
-  if (M < 1 || M > 32 || (K % 32) != 0 || N < 1 || (epi != EPI_RESIDUAL && epi != EPI_GELU && epi != EPI_QKV)) return cudaErrorInvalidValue;
+  if (M < 1 || M > 64 || (K % 32) != 0 || N < 1 || (epi != EPI_RESIDUAL && epi != EPI_GELU && epi != EPI_QKV)) return cudaErrorInvalidValue;
   if ((epi == EPI_GELU && out_lo == nullptr) || (epi == EPI_QKV && qkv == nullptr)) return cudaErrorInvalidValue;
   cudaError_t e = prepare_decode();
   if (e != cudaSuccess) return e;
@@ -610,8 +634,11 @@ cudaError_t launch_stream_gemm(const __nv_bfloat16* x, const __nv_bfloat16* x_lo
   if (qkv != nullptr) qd = *qkv;
   const int kind = epi == EPI_RESIDUAL ? SO_ADD : epi == EPI_GELU ? SO_GELU : SO_QKV;
   // up to 16 rows: 16 features a CTA; beyond, every CTA's own copy of the activations (2 M K or 4 M K bytes from L2) asks for 32
-  const int cg = M <= 8 ? 1 : M <= 16 ? 2 : M <= 24 ? 3 : 4;
-  const int R = cg <= 2 ? 16 : 32, tiles = (N + R - 1) / R, all = K / 32;
+  const int cg = M <= 8 ? 1 : M <= 16 ? 2 : M <= 24 ? 3 : M <= 32 ? 4 : M <= 40 ? 5 : M <= 48 ? 6 : 8;
+  // and for 48 where 32 would make more CTAs than SMs (XL verification of 33 rows: 3.03 -> 2.94 ms; where 32 features fill one
+  // wave, 48 only idle SMs: 12 layers of width 768, 33 rows 0.54 -> 0.58 ms).  Additive products have K shares to fill the chip.
+  const bool mt3 = cg >= 3 && cg <= 6 && kind != SO_ADD && (N + 31) / 32 > SMS;
+  const int R = cg <= 2 ? 16 : mt3 ? 48 : 32, tiles = (N + R - 1) / R, all = K / 32;
   int ks = 1;
   if (kind == SO_ADD) {
     // K shares: about two CTAs an SM, at least 8 slices of 32 (one a warp) each, and three CTAs an SM in shared memory
@@ -639,8 +666,11 @@ cudaError_t launch_stream_gemm(const __nv_bfloat16* x, const __nv_bfloat16* x_lo
   switch (cg) {
     case 1: return go(stream_kernel<1, 1, false>, stream_kernel<1, 1, true>);
     case 2: return go(stream_kernel<1, 2, false>, stream_kernel<1, 2, true>);
-    case 3: return go(stream_kernel<2, 3, false>, stream_kernel<2, 3, true>);
-    default: return go(stream_kernel<2, 4, false>, stream_kernel<2, 4, true>);
+    case 3: return mt3 ? go(stream_kernel<3, 3, false>, stream_kernel<3, 3, true>) : go(stream_kernel<2, 3, false>, stream_kernel<2, 3, true>);
+    case 4: return mt3 ? go(stream_kernel<3, 4, false>, stream_kernel<3, 4, true>) : go(stream_kernel<2, 4, false>, stream_kernel<2, 4, true>);
+    case 5: return mt3 ? go(stream_kernel<3, 5, false>, stream_kernel<3, 5, true>) : go(stream_kernel<2, 5, false>, stream_kernel<2, 5, true>);
+    case 6: return mt3 ? go(stream_kernel<3, 6, false>, stream_kernel<3, 6, true>) : go(stream_kernel<2, 6, false>, stream_kernel<2, 6, true>);
+    default: return go(stream_kernel<2, 8, false>, stream_kernel<2, 8, true>);
   }
 }
 
@@ -651,11 +681,11 @@ cudaError_t launch_attn_few(const __nv_bfloat16* q, int q_ld, const __nv_bfloat1
   if (e != cudaSuccess) return e;
   FewParams p;
   p.q = q; p.q_ld = q_ld; p.kc = kc; p.vt = vt; p.out = out; p.ctx_len = ctx_len; p.R = R; p.n_ctx = n_ctx; p.d = n_head * 64;
-  p.splits = key_splits;
-  while (p.splits > 1 && n_head * batch * p.splits > SMS) p.splits >>= 1;       // one CTA an SM
+  p.groups = (R + TOK - 1) / TOK;
+  p.splits = attn_few_splits(batch, R, n_head, key_splits);
   p.s_ld = scores_ld(n_ctx, p.splits);
-  const dim3 grid(n_head * p.splits, batch), block(32 * AT_WARPS);
-  const size_t smem = attn_smem(R, n_ctx, p.splits);
+  const dim3 grid(n_head * p.splits, batch * p.groups), block(32 * AT_WARPS);
+  const size_t smem = attn_smem(R < TOK ? R : TOK, n_ctx, p.splits);
   auto go = [&](auto kernel) {
     if (p.splits > 1) return launch_k_cluster(kernel, grid, block, smem, st, (unsigned)p.splits, p);
     return launch_k(kernel, grid, block, smem, st, p);

@@ -159,6 +159,7 @@ cudaError_t launch_attn_tc(const __nv_bfloat16* q, long long q_rows_total, int q
 // ---- forwards of a few token rows, bf16, d_head 64 (sdd_decode.cu) -----------------------------
 bool few_rows_fit(int M, int d, int d_head);
 bool attn_few_fits(int R, int n_ctx);
+int attn_few_splits(int batch, int R, int n_head, int key_splits);
 cudaError_t prepare_decode();
 // M = 1 or 2: out = epilogue(LayerNorm(h) W^T + bias); qkv given: Q to out (row stride N), K and V^T to the caches (verify
 // positions); else GELU as a hi/lo pair to out / out_lo (row stride N)

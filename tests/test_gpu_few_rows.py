@@ -51,3 +51,14 @@ def test_verification_rows(plens, gamma):
     ref, slots_ref = _logits("0", 5, plens, gamma, "round")
     assert np.array_equal(slots, slots_ref)          # the drafts do not depend on the target's path
     assert np.abs(few - ref).max() < 2e-2 and np.linalg.norm(few - ref) < 1e-2 * np.linalg.norm(ref)
+
+
+# column groups of 5, 6 and 8, 48-feature CTAs (width 1600 from 17 rows on), the row limits of both widths, row groups of 8
+@pytest.mark.parametrize("heads", [5, 25])
+@pytest.mark.parametrize("plens,gamma", [([100], 16), ([300], 32), ([40, 190, 2], 12), ([400], 40), ([100, 333, 7], 15), ([200], 48),
+                                         ([31], 63), ([250, 9, 63, 64], 15)])
+def test_verification_rows_wide(heads, plens, gamma):
+    few, slots = _logits("64", heads, plens, gamma, "round")
+    ref, slots_ref = _logits("0", heads, plens, gamma, "round")
+    assert np.array_equal(slots, slots_ref)
+    assert np.abs(few - ref).max() < 2e-2 and np.linalg.norm(few - ref) < 1e-2 * np.linalg.norm(ref)
