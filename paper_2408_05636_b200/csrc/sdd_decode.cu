@@ -308,7 +308,7 @@ stream_kernel(const __nv_bfloat16* x, const __nv_bfloat16* x_lo, const __nv_bflo
     }
   };
   // slices whose activations are in flight together (more of them spill: 8 at one column group cost 0.1 ms of a 1.2 ms step)
-  constexpr int NB = MT == 3 ? (CG <= 4 ? 3 : CG <= 6 ? 2 : 1) : CG == 1 ? 4 : CG == 2 ? (LO ? 2 : 4) : CG <= 4 ? 2 : 1;
+  constexpr int NB = MT == 3 ? (CG <= 4 ? 3 : CG <= 6 ? 2 : 1) : CG == 1 ? 4 : CG == 2 ? (LO ? 2 : 4) : CG == 5 && LO ? 1 : 2;
   bool ok = true, waited = false;
   for (int i0 = warp; i0 < n_sl; i0 += WARPS * NB) {
     uint4 hi[NB][CG], lo[LO ? NB : 1][LO ? CG : 1];
